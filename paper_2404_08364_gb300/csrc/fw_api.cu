@@ -424,6 +424,7 @@ extern "C" int fw_walk_ex(fw_graph* G, int32_t algo, const fw_params* p, const i
     r.n_q = n_q;
     r.q_begin = 0;
     r.q_id0 = q_id0;
+    tab.algos = 1u << algo;
 
     // classify buffers; host ones are staged through device memory
     const int64_t width = (int64_t)max_len + 1;
@@ -527,6 +528,7 @@ extern "C" int fw_walk_multi(fw_graph* G, const fw_request* reqs, int32_t n_req,
         r.q_begin = total;
         r.q_id0 = q.q_id0;
         total += q.n_q;
+        tab.algos |= 1u << q.algo;
     }
     if (total == 0) return FW_OK;
     return launch(G, mode, tab, n_req, total, (cudaStream_t)stream);
@@ -652,6 +654,7 @@ extern "C" int fw_walk_noalloc(fw_graph* G, const fw_request* reqs, int32_t n_re
         g_noalloc_addr[G->device] = dev;
     }
     int64_t total = 0;
+    uint32_t algos = 0;
     const int mode = reqs[0].params.mode;
     for (int i = 0; i < n_req; ++i) {
         const fw_request& q = reqs[i];
@@ -675,6 +678,7 @@ extern "C" int fw_walk_noalloc(fw_graph* G, const fw_request* reqs, int32_t n_re
         r.q_begin = total;
         r.q_id0 = q.q_id0;
         total += q.n_q;
+        algos |= 1u << q.algo;
     }
     if (total == 0) return FW_OK;
     cudaStream_t st = (cudaStream_t)stream;
@@ -687,6 +691,7 @@ extern "C" int fw_walk_noalloc(fw_graph* G, const fw_request* reqs, int32_t n_re
     ReqTable tab;
     memset(&tab, 0, sizeof tab);
     tab.ext = dev->reqs;
+    tab.algos = algos;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cap);
     const bool timed = cap == cudaStreamCaptureStatusNone;

@@ -130,6 +130,7 @@ extern "C" int fw_walk_batched(fw_graph* g, int32_t algo, const fw_params* p, co
         chk(cudaMemcpyAsync(&q.scratch->cursor, h_zero, sizeof(unsigned long long), cudaMemcpyHostToDevice, q.st));
         ReqTable tab;
         memset(&tab, 0, sizeof tab);
+        tab.algos = 1u << algo;
         ReqDev& r = tab.r[0];
         r = base;
         r.starts = q.starts;

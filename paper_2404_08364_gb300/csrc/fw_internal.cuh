@@ -25,15 +25,10 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
             k.x += 0x9E3779B9u;
             k.y += 0xBB67AE85u;
         }
-#ifdef __CUDA_ARCH__
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-#else
-        const uint32_t hi0 = (uint32_t)(((uint64_t)0xD2511F53u * c.x) >> 32);
-        const uint32_t hi1 = (uint32_t)(((uint64_t)0xCD9E8D57u * c.z) >> 32);
-#endif
-        const uint32_t lo0 = 0xD2511F53u * c.x;
-        const uint32_t lo1 = 0xCD9E8D57u * c.z;
+        // one widening multiplication gives both halves
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
+        const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
         c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
     }
     return c;
@@ -119,6 +114,8 @@ static_assert(sizeof(Scratch) == 128, "scratch layout");
 constexpr int kMaxInlineReqs = 16;
 struct ReqTable {
     const ReqDev* ext;
+    uint32_t algos;  // algorithms among the requests (bit FW_WEIGHTED ..)
+    uint32_t pad;
     ReqDev r[kMaxInlineReqs];
 };
 
@@ -170,6 +167,10 @@ inline cudaError_t launch_walk(const GraphDev& g, int mode, const ReqTable& reqs
 // fw_walk.cu.
 cudaError_t launch_serve(const GraphDev& g, int mode, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
                          cudaStream_t stream);
+
+// The fast-mode launch of requests without node2vec (fw_fast.cu).
+cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                        unsigned long long* counters, const Tuning& tune, cudaStream_t stream);
 
 Tuning default_tuning();
 Tuning sanitize_tuning(Tuning t);

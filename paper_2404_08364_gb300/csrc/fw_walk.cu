@@ -1867,6 +1867,8 @@ cudaError_t launch_walk(const GraphDev& g, int mode, const ReqTable& reqs, int n
     const Tuning tu = sanitize_tuning(tune);
     if (total <= 0) return cudaSuccess;
     const bool exact = mode == FW_EXACT;
+    if (!exact && !(reqs.algos >> FW_NODE2VEC & 1u))
+        return launch_fast(g, reqs, n_req, total, cursor, counters, tu, stream);
     switch (tu.block_threads) {
         case 128:
             return exact ? launch_one<MODE_EXACT, 128>(g, reqs, n_req, total, cursor, counters, tu, stream)

@@ -1,0 +1,73 @@
+"""One-step laws of rows whose lengths sit at the edges of the kernels' tiles
+(quads, 128-entry halves, 256-entry stages, 512-entry pairs, 1024-entry
+chunks, 16384-entry segments), at many alignments, the last row ending at the
+end of arrays whose size is no multiple of 16.
+
+Fast mode: 2^16 draws per row against w_i / sum(w), chi-square p > 1e-6 (about
+100 rows and rules in all, so a false alarm has a chance below 1e-4)."""
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_common import built, chi2_tv, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+LENS = (1, 2, 3, 15, 16, 17, 31, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 1537, 4101, 16383,
+        16384, 16385, 20003)
+N = 1 << 16
+P_MIN = 1e-6
+
+
+class _G:
+    pass
+
+
+def edge_graph(lens=LENS, n=60000, seed=3):
+    """Vertex i < len(lens) has a sorted random row of lens[i] entries."""
+    rng = np.random.default_rng(seed)
+    g = _G()
+    g.n = n
+    cols = [np.sort(rng.choice(n, k, replace=False)) for k in lens]
+    g.row_ptr = np.zeros(n + 1, dtype=np.int64)
+    g.row_ptr[1:len(lens) + 1] = np.cumsum(lens)
+    g.row_ptr[len(lens) + 1:] = g.row_ptr[len(lens)]
+    g.col = np.concatenate(cols).astype(np.int32)
+    g.m = g.col.size
+    g.w_u32 = rng.integers(1, 1000, g.m).astype(np.uint32)
+    g.w_f32 = g.w_u32.astype(np.float32)
+    g.etype = rng.integers(0, 5, g.m).astype(np.int8)
+    return g
+
+
+def load(g):
+    need_gpu()
+    built()
+    from paper_2404_08364_gb300 import DeviceGraph
+    t = [torch.from_numpy(x) for x in (g.row_ptr, g.col, g.w_f32, g.w_u32.view(np.int32), g.etype)]
+    return DeviceGraph.from_tensors(*t, borrow=True)
+
+
+@pytest.mark.parametrize("algo", ["weighted", "metapath", "ppr"])
+@pytest.mark.parametrize("d_warp", [0, 1024])
+def test_fast_laws_at_tile_edges(algo, d_warp):
+    g = edge_graph()
+    assert g.m % 16 and g.m % 4
+    dg = load(g)
+    if d_warp:
+        dg.set_tuning(d_warp=d_warp)  # the longer rows go to the CTA sampler
+    starts = torch.arange(len(LENS), dtype=torch.int32, device="cuda").repeat_interleave(N)
+    paths, plen = dg.walk(algo, starts, 1, 20240501 + d_warp, mode="fast", schema=(2,), ppr_stop=0.5)
+    dg.stats()
+    nxt = paths[:, 1].view(len(LENS), N).cpu().numpy()
+    for i, d in enumerate(LENS):
+        row = slice(int(g.row_ptr[i]), int(g.row_ptr[i + 1]))
+        w = g.w_f32[row].astype(np.float64) * (g.etype[row] == 2 if algo == "metapath" else 1)
+        if w.sum() == 0:
+            assert (nxt[i] == -1).all(), d
+            continue
+        at = np.searchsorted(g.col[row], nxt[i])
+        assert (at < d).all() and (g.col[row][at] == nxt[i]).all(), (algo, d)
+        _, p = chi2_tv(np.bincount(at, minlength=d), w / w.sum(), N)
+        assert p > P_MIN, (algo, d, p)
