@@ -85,7 +85,7 @@ __device__ __forceinline__ float unit_open(uint32_t w) {
 }
 
 // First index i >= pos with B[i] >= x, or pd.  Warp-collective, uniform result.
-__device__ __forceinline__ int lower_bound_from(const int32_t* __restrict__ B, int pd, int pos, int x, int lane) {
+__device__ __noinline__ int lower_bound_from(const int32_t* __restrict__ B, int pd, int pos, int x, int lane) {
     {
         const int idx = pos + lane;
         const int v = idx < pd ? __ldg(B + idx) : INT_BIG;

@@ -54,36 +54,29 @@ constexpr int NSEG_MAX = 64;      // segments per hub task
 constexpr int kSegQuads = 4096;
 constexpr int STAGE = 256;             // entries per reservoir stage: two 128-entry halves, a quad of each per lane
 constexpr int PAIR = 2 * STAGE;        // entries of one scan iteration
+constexpr int CHUNK = 1024;            // node2vec: columns staged (and tested) at a time
+// node2vec: a chunk of n entries whose window holds more than kDenseRatio n +
+// kDenseMin further values of N(prev) is searched from its own side.  Measured
+// (R-MAT-20 / R-MAT-25 batches, ms): 1 n + 128: 39.8 / 203; 2 n + 256: 39.2 /
+// 202; 3 n + 512: 37.8 / 198.6; 4 n + 1024: 37.2 / 198.3.
+constexpr int kDenseRatio = 4, kDenseMin = 1024;
+constexpr int NSPL = 128;              // node2vec: splitters of a dense window
+constexpr int kSplCap = 154;           // their search reads up to here
 constexpr int ST_EMPTY = 0, ST_READY = 1, ST_HUB = 2, ST_FINISH = 3;
 // hub task control word: state << 24 | segments << 16 | next segment to hand out
 constexpr unsigned H_FREE = 0u, H_SETUP = 1u << 24, H_ACTIVE = 2u << 24, H_STATE = 0xFFu << 24;
 __device__ __forceinline__ int hub_nseg(unsigned ctl) { return (int)(ctl >> 16 & 0xFFu); }
 __device__ __forceinline__ int hub_next(unsigned ctl) { return (int)(ctl & 0xFFFFu); }
 
-// Per-step view of one walk, held in registers by the lanes of its sampler.
-struct StepCtx {
-    long long beg;
-    long long pbeg;
-    int d;
-    int pdeg;
-    int prev;
-    int algo;
-    int want;   // MetaPath label for this move
-    float f0, f1, f2;  // node2vec factors: return, in, out
-};
-
-// A CTA hub task: one step of one walk whose row is longer than d_t.
+// A CTA hub task: one step of one walk whose row is longer than d_t.  The
+// step itself is what the owner's slot says (it does not change until the
+// task is done).
 struct HubTask {
     unsigned ctl;     // one atomic claims a segment and tells whether the task
                       // was live and how many segments it has
     int slot;         // owner slot (index into the CTA's slots)
-    int seg_e;        // entries per segment
     int done_seg;
     unsigned long long best;  // (race-time bits << 32) | row index
-    StepCtx c;
-    uint64_t seed;
-    uint64_t qid;
-    uint32_t t;
 };
 
 struct __align__(16) Slot {
@@ -103,14 +96,23 @@ struct CtaHead {
 // Per-warp shared memory.
 struct WarpHead {
     unsigned long long cnt[C_NUM];
+    unsigned long long idle_since;  // when the warp ran out of work (0: it has some)
+    unsigned nap;                   // idle back-off (ns)
+    int exhausted;                  // no query is left to claim
 };
 constexpr int kHeadBytes = (sizeof(CtaHead) + 127) & ~127;
 constexpr int kWarpHeadBytes = (sizeof(WarpHead) + 127) & ~127;
 
-// Offsets inside a warp's area.
+// Offsets inside a warp's area.  node2vec: a chunk's columns (and one word
+// that equals no vertex id), its membership bytes, the splitters of a dense
+// window, the barrier of the columns' copies.
 template <bool N2V>
 struct Area {
-    static constexpr int HEAD = 0;
+    static constexpr int COL = 0;
+    static constexpr int MASK = COL + (N2V ? CHUNK * 4 + 16 : 0);
+    static constexpr int SPL = MASK + (N2V ? CHUNK : 0);
+    static constexpr int BAR = SPL + (N2V ? kSplCap * 4 : 0);
+    static constexpr int HEAD = (BAR + (N2V ? 8 : 0) + 127) & ~127;
     static constexpr int BYTES = HEAD + kWarpHeadBytes;
 };
 
@@ -166,19 +168,13 @@ __device__ __forceinline__ int seg_entries(int r_a, int d) {
     return (int)(((sq + 31) & ~31u) << 2);
 }
 
-// What the draws of one segment are keyed by.
-struct Stream {
-    uint64_t seed, qid;
-    uint32_t t, id;
-};
-
 // Find every record inside a stage, in visiting order (lane by lane, j
 // ascending: any fixed order gives the same law), and leave R with the skip
 // budget past the stage.  The stage starts at row index e0; w: this lane's
 // entries (0: outside the row or excluded), row indices e0 + 4 lane + j
 // (j < 4) and e0 + 4 lane + 124 + j (j >= 4); own: their sum.
 __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float own, int e0, int lane,
-                                              const Stream& S) {
+                                              const Slot& sl, int stream) {
     float incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -224,7 +220,8 @@ __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float
         if (lane < L) live = 0u;
         if (lane == L) live = live >> (jj + 1) << (jj + 1);
         if (R.i == R.have) {
-            const uint4 o = lane_block(S.seed, S.qid, S.t, S.id, (uint32_t)(R.i + lane) >> 1);
+            const uint4 o = lane_block(sl.rq.seed, (uint64_t)(sl.rq.q_id0 + sl.q), (uint32_t)sl.t, (uint32_t)stream,
+                                       (uint32_t)(R.i + lane) >> 1);
             R.u1 = unit_open(lane & 1 ? o.z : o.x);
             R.nl2 = -__logf(unit_open(lane & 1 ? o.w : o.y));
             R.have += 32;
@@ -249,7 +246,8 @@ __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float
 // A stage's total is the xor butterfly sum of its lanes' sums (the same in
 // every lane, as a + b = b + a in IEEE arithmetic); the two butterflies share
 // their last four steps, one stage in each half of the warp.
-__device__ __forceinline__ void offer_pair(Res& R, const float (&w)[16], bool two, int e0, int lane, const Stream& S) {
+__device__ __forceinline__ void offer_pair(Res& R, float (&w)[16], bool two, int e0, int lane, const Slot& sl,
+                                           int stream) {
     const float own0 = ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
     const float own1 = ((w[8] + w[9]) + (w[10] + w[11])) + ((w[12] + w[13]) + (w[14] + w[15]));
     const bool up = lane & 16;
@@ -270,95 +268,376 @@ __device__ __forceinline__ void offer_pair(Res& R, const float (&w)[16], bool tw
         R.Xl = al + ((a - b) - t1);
         return;
     }
+    float tot = t0, own = own0;
 #pragma unroll 1
-    for (int h = 0; h < (two ? 2 : 1); ++h) {
-        const float tot = h ? t1 : t0;
+    for (;;) {
         if (R.Xh - tot + R.Xl > 0.0f) {
             const float s = R.Xh - tot;
             R.Xl += (R.Xh - s) - tot;
             R.Xh = s;
-            continue;
+        } else {
+            const float ws[8] = {w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]};
+            stage_records(R, ws, own, e0, lane, sl, stream);
         }
-        float ws[8];
+        if (!two) return;
+        two = false;
+        // the second stage takes the first one's place (moved, not indexed:
+        // an index would put w in local memory)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) ws[j] = h ? w[8 + j] : w[j];
-        stage_records(R, ws, h ? own1 : own0, e0 + h * STAGE, lane, S);
+        for (int j = 0; j < 8; ++j) w[j] = w[8 + j];
+        e0 += STAGE;
+        tot = t1;
+        own = own1;
     }
+}
+
+// One lane's quad at row index rel whose last entries lie past the end of the
+// arrays (`left` entries of the row's base to their end).  Out of line: it
+// runs for the graph's last row only.
+__device__ __noinline__ float4 load_quad_tail(const float* wrow, int rel, int left) {
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (rel < left) v.x = __ldg(wrow + rel);
+    if (rel + 1 < left) v.y = __ldg(wrow + rel + 1);
+    if (rel + 2 < left) v.z = __ldg(wrow + rel + 2);
+    return v;
+}
+__device__ __noinline__ int load_labels_tail(const int8_t* lrow, int rel, int left) {
+    int l = 0;
+    for (int j = 0; j < 4 && rel + j < left; ++j) l |= (int)(uint8_t)__ldg(lrow + rel + j) << (8 * j);
+    return l;
 }
 
 // This lane's quads of a pair whose first entry is row index r0, weights with
-// MetaPath's label rule applied; 0 outside the row indices [0, lim).  Only an
-// edge pair (the range's first or last) holds such entries; its quads are
-// loaded one by one, so that nothing past the end of the arrays is read.
-// wrow, lrow: the row's first weight and label.
+// MetaPath's label rule applied; 0 outside the row indices [0, lim) (only an
+// edge pair, the range's first or last, holds such entries).  wrow, lrow: the
+// row's first weight and label.
+template <bool LAB>
 __device__ __forceinline__ void load_pair(const float* __restrict__ wrow, const int8_t* __restrict__ lrow, int want,
                                           int r0, int lim, int left, int lane, float (&w)[16]) {
     const int at = r0 + 4 * lane;
+    const float4* q = reinterpret_cast<const float4*>(wrow + at);
+    const int* ql = reinterpret_cast<const int*>(lrow + at);
+    int l[4] = {0, 0, 0, 0};
     if (r0 >= 0 && r0 + PAIR <= lim) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(wrow + at) + k * 32);
+            const float4 v = __ldg(q + 32 * k);
             w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
         }
-        if (lrow) {
-            int l[4];
+        if (LAB && lrow) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) l[k] = __ldg(reinterpret_cast<const int*>(lrow + at) + k * 32);
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                if ((int)(int8_t)(l[j >> 2] >> (8 * (j & 3))) != want) w[j] = 0.0f;
+            for (int k = 0; k < 4; ++k) l[k] = __ldg(ql + 32 * k);
         }
-        return;
-    }
+    } else {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[4 * k + j] = 0.0f;
-        if (r0 + 128 * k >= lim) continue;  // the whole warp's quads lie past the range
-        const int rel = at + 128 * k;       // row index of the quad's first entry
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        int l = 0;
-        if (rel + 4 <= left) {
+        for (int k = 0; k < 4; ++k) {
+            const int rel = at + 128 * k;
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (rel < lim) {
-                v = __ldg(reinterpret_cast<const float4*>(wrow + rel));
-                if (lrow) l = __ldg(reinterpret_cast<const int*>(lrow + rel));
+                if (rel + 4 <= left) {
+                    v = __ldg(q + 32 * k);
+                    if (LAB && lrow) l[k] = __ldg(ql + 32 * k);
+                } else {
+                    v = load_quad_tail(wrow, rel, left);
+                    if (LAB && lrow) l[k] = load_labels_tail(lrow, rel, left);
+                }
             }
-        } else if (rel < lim) {
-            // the last quad of arrays whose size is no multiple of 4
-            const int some = left - rel;
-            v.x = __ldg(wrow + rel);
-            if (some > 1) v.y = __ldg(wrow + rel + 1);
-            if (some > 2) v.z = __ldg(wrow + rel + 2);
-            if (lrow)
-                for (int j = 0; j < some; ++j) l |= (int)(uint8_t)__ldg(lrow + rel + j) << (8 * j);
+            w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
         }
-        const float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if ((unsigned)(rel + j) < (unsigned)lim) w[4 * k + j] = x[j];
-        if (lrow) {
+        for (int j = 0; j < 16; ++j)
+            if ((unsigned)(at + 128 * (j >> 2) + (j & 3)) >= (unsigned)lim) w[j] = 0.0f;
+    }
+    if (LAB && lrow) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if ((int)(int8_t)(l >> (8 * j)) != want) w[4 * k + j] = 0.0f;
-        }
+        for (int j = 0; j < 16; ++j)
+            if ((int)(int8_t)(l[j >> 2] >> (8 * (j & 3))) != want) w[j] = 0.0f;
     }
 }
 
-// Scan the entries of row indices [r_a, lim) of c's row (r_a a multiple of 16
-// in the CSR arrays, down to -15): weights with the rule's factors, offered
-// to the warp's reservoir R.  Warp-collective.
-template <bool N2V>
-__device__ __forceinline__ void scan_range(const GraphDev& g, const StepCtx& c, int r_a, int lim, int lane, Res& R,
-                                           const Stream& S) {
-    const float* wrow = g.w_f32 + c.beg;
-    const int8_t* lrow = c.algo == FW_METAPATH ? g.etype + c.beg : nullptr;
-    const int left = (int)min((long long)INT_BIG, g.m - c.beg);  // entries up to the end of the arrays
-#pragma unroll 1
-    for (int r0 = r_a; r0 < lim; r0 += PAIR) {
-        float w[16];
-        load_pair(wrow, lrow, c.want, r0, lim, left, lane, w);
-        offer_pair(R, w, r0 + STAGE < lim, r0, lane, S);
+// --------------------------------------------------------------------------
+// node2vec membership: which entries of a chunk of N(cur) are also in
+// N(prev) = B?  Both rows ascend.  The values of B inside the chunk's range are
+// taken 128 at a time, four per lane, and each is located in the staged columns
+// by a binary search; a hit sets its entry's byte (the values of B are
+// distinct, so no two lanes write one byte).
+//
+// The four searches of a lane run in lockstep: a step is one shared load, one
+// compare and one predicated add each, and the loads of the four overlap.  The
+// steps are uneven (489, 251, 131, ...) because even ones put a warp's probes
+// on few banks (p + 2^k - 1 with p a multiple of 2^(k+1)); r entries take
+// steps s with r -> max(r - s, s - 1), here 1024, 535, 284, 153, 86, 49, 26,
+// 13, 6, 3, 1, 0.
+// --------------------------------------------------------------------------
+
+template <int OFF>
+__device__ __forceinline__ int lds_at(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.b32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
+    return v;
+}
+
+template <int S, int NV>
+__device__ __forceinline__ void lb_step(uint32_t (&a)[NV], const int (&x)[NV]) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+        if (lds_at<(S - 1) * 4>(a[i]) < x[i]) a[i] += S * 4;
+}
+
+// Move each a[i] from the first staged column to the first that is >= x[i].
+// n columns are staged, with values above every x up to staged_cap(n).
+template <int NV>
+__device__ __forceinline__ void lb_search(uint32_t (&a)[NV], const int (&x)[NV], int n) {
+    if (n > 535) lb_step<489>(a, x);
+    if (n > 284) lb_step<251>(a, x);
+    lb_step<131>(a, x);
+    lb_step<67>(a, x);
+    lb_step<37>(a, x);
+    lb_step<23>(a, x);
+    lb_step<13>(a, x);
+    lb_step<7>(a, x);
+    lb_step<3>(a, x);
+    lb_step<2>(a, x);
+    lb_step<1>(a, x);
+}
+__device__ __forceinline__ int staged_cap(int n) { return n > 535 ? CHUNK : (n > 284 ? 536 : 288); }
+
+// Four 32-entry blocks of B from `base` in one round trip (INT_BIG past pd).
+__device__ __forceinline__ void load_b128(const int32_t* __restrict__ B, int pd, int base, int lane, int (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int idx = base + 32 * i + lane;
+        v[i] = idx < pd ? __ldg(B + idx) : INT_BIG;
     }
+}
+
+// Dense windows: B holds more values inside the chunk's range than the chunk
+// has entries, so each staged entry x > `above` (entries [ia, n)) searches the
+// window B[from, end) instead.  NSPL splitters B[from + (s+1) w - 1] (w =
+// ceil((end - from) / NSPL)) are staged; x's lower bound lies in the bracket
+// after the splitters below x, and a binary search of that bracket in global
+// memory finishes it, four entries per lane in lockstep.  Warp-collective.
+__device__ __noinline__ void dense_members(const int32_t* __restrict__ B, int end, int from, int above,
+                                           unsigned char* __restrict__ area, int ia, int n, int lane) {
+    const int* col = reinterpret_cast<const int*>(area + Area<true>::COL);
+    int* spl = reinterpret_cast<int*>(area + Area<true>::SPL);
+    const uint32_t sa = smem_u32(spl);
+    const int w = (end - from + NSPL - 1) / NSPL;
+#pragma unroll 1
+    for (int i = lane; i < kSplCap; i += 32)
+        spl[i] = i < NSPL ? __ldg(B + min((long long)from + (long long)(i + 1) * w - 1, (long long)end - 1)) : INT_BIG;
+    __syncwarp();
+#pragma unroll 1
+    for (int e0 = lane; e0 < n; e0 += 128) {
+        int x[4], a[4], b[4];
+        uint32_t s[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int e = e0 + 32 * j;
+            x[j] = e >= ia && e < n ? col[e] : -1;
+            s[j] = sa;
+        }
+        // (splitters below x: 153 entries are searched, INT_BIG from NSPL on)
+        lb_step<67>(s, x);
+        lb_step<37>(s, x);
+        lb_step<23>(s, x);
+        lb_step<13>(s, x);
+        lb_step<7>(s, x);
+        lb_step<3>(s, x);
+        lb_step<2>(s, x);
+        lb_step<1>(s, x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = x[j] > above ? (int)min((long long)from + (long long)((s[j] - sa) >> 2) * w, (long long)end) : end;
+            b[j] = (int)min((long long)a[j] + w, (long long)end);
+        }
+        bool more = true;
+#pragma unroll 1
+        while (more) {
+            more = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (a[j] < b[j]) {
+                    more = true;
+                    const int mid = (int)(((unsigned)a[j] + (unsigned)b[j]) >> 1);
+                    if (__ldg(B + mid) < x[j]) a[j] = mid + 1;
+                    else b[j] = mid;
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (a[j] < end && __ldg(B + a[j]) == x[j]) area[Area<true>::MASK + e0 + 32 * j] = 1;
+    }
+    __syncwarp();  // the splitters are rewritten by the next dense chunk
+}
+
+// Set the membership bytes of a chunk: staged entries [ia, n) of range [amin,
+// amax].  pos: cursor into B, every value before it lies below the chunk.
+// Returns the smallest value of B above amax (INT_MIN: not known).
+// Warp-collective.
+__device__ __forceinline__ int chunk_members(const int32_t* __restrict__ B, int pd, int& pos, int amin, int amax, int ia,
+                                             int n, unsigned char* __restrict__ area, int lane) {
+    const uint32_t col = smem_u32(area + Area<true>::COL), mask = smem_u32(area + Area<true>::MASK);
+    uint4* m4 = reinterpret_cast<uint4*>(area + Area<true>::MASK);
+    m4[lane] = make_uint4(0u, 0u, 0u, 0u);
+    m4[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    int v[4];
+    load_b128(B, pd, pos, lane, v);
+    int last = __shfl_sync(FULL, v[3], 31);
+    if (last < amin) {
+        // the whole block lies below this chunk: jump to the chunk's range
+        pos = lower_bound_from(B, pd, pos + 128, amin, lane);
+        load_b128(B, pd, pos, lane, v);
+        last = __shfl_sync(FULL, v[3], 31);
+    }
+    bool checked = false;
+#pragma unroll 1
+    while (pos < pd) {
+        int nv[4];
+        load_b128(B, pd, pos + 128, lane, nv);  // lands while this block is searched
+        uint32_t a[4] = {col, col, col, col};
+        lb_search(a, v, n);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (lds_at<0>(a[i]) == v[i])
+                asm volatile("st.shared.u8 [%0], %1;" ::"r"(mask + ((a[i] - col) >> 2)), "r"(1) : "memory");
+        if (last > amax) {
+            int nb = INT_BIG;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (v[i] > amax) nb = min(nb, v[i]);
+            return __reduce_min_sync(FULL, nb);
+        }
+        const int first = __shfl_sync(FULL, v[0], 0);
+        pos += 128;
+        // When, at this block's density, B holds kDenseRatio times as many
+        // further values in the chunk's range as the chunk has entries, look
+        // where they end and search from the chunk's side.
+        const int dense = kDenseRatio * n + kDenseMin;
+        if (!checked && (float)(amax - last) * 128.0f > (float)dense * (float)(last - first + 1)) {
+            checked = true;
+            const int ub = lower_bound_from(B, pd, pos, amax + 1, lane);
+            if (ub - pos > dense) {
+                dense_members(B, ub, pos, last, area, ia, n, lane);
+                pos = ub;
+                return INT_MIN;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = nv[i];
+        last = __shfl_sync(FULL, v[3], 31);
+    }
+    return INT_BIG;
+}
+
+// Scan the entries of row indices [r_a, lim) of slot sl's row (r_a a multiple
+// of 16 in the CSR arrays, down to -15) as random stream `stream`: weights with
+// the rule's factors, offered to the warp's reservoir R.  False if a copy never
+// landed.  Warp-collective.
+template <bool N2V, bool LAB>
+__device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, int r_a, int lim, int lane,
+                                           unsigned char* area, uint32_t& ph, Res& R, int stream) {
+    const long long beg = sl.row[0];
+    const float* wrow = g.w_f32 + beg;
+    const int algo = sl.rq.algo;
+    const int8_t* lrow = nullptr;
+    int want = 0;
+    if (LAB && algo == FW_METAPATH) {
+        lrow = g.etype + beg;
+        want = (int)sl.rq.schema[(uint32_t)sl.t % (uint32_t)sl.rq.schema_len];
+    }
+    const int left = (int)min(0x7fffff00ll, g.m - beg);  // entries up to the end of the arrays
+    const int prev = N2V ? sl.prev : -1;
+    const bool n2v = N2V && algo == FW_NODE2VEC && prev >= 0;
+    const int32_t* B = N2V ? g.col + sl.pbeg : nullptr;
+    int pos = -1, nb = INT_MIN;
+    int* col = reinterpret_cast<int*>(area + Area<N2V>::COL);
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(area + Area<N2V>::BAR);
+    // whole 16-entry groups inside the arrays, as copies take them
+    const int whole = r_a + ((left - r_a) & ~15);
+    if (n2v && lane == 0) {
+        const int k = min(min(CHUNK, (lim - r_a + 15) & ~15), whole - r_a);
+        mbar_arrive_expect_tx(bar, (uint32_t)k * 4u);
+        if (k > 0) tma_load_1d(col, g.col + beg + r_a, (uint32_t)k * 4u, bar);
+    }
+#pragma unroll 1
+    for (int r0 = r_a; r0 < lim; r0 += N2V ? CHUNK : PAIR) {
+        bool some = false;
+        int prevpos = -1;
+        if (n2v) {
+            if (!mbar_wait_warp(bar, ph)) return false;
+            ph ^= 1u;
+            // staged entries [ia, n) belong to the row; the others take values
+            // that keep the chunk ascending and equal no vertex id
+            const int ia = max(0, -r0), n = min(CHUNK, lim - r0);
+            bool wrote = false;
+            if (whole < r0 + n) {
+#pragma unroll 1
+                for (int e = max(whole - r0, 0) + lane; e < n; e += 32) col[e] = __ldg(g.col + beg + r0 + e);
+                wrote = true;
+            }
+            const int cap = staged_cap(n);
+            if (ia > 0 || n < cap) {
+                if (lane < ia) col[lane] = INT_MIN;
+                const int n4 = (n + 3) & ~3;
+                if (n + lane < n4) col[n + lane] = INT_BIG;
+#pragma unroll 1
+                for (int e = n4 + 4 * lane; e < cap; e += 128)
+                    *reinterpret_cast<int4*>(col + e) = make_int4(INT_BIG, INT_BIG, INT_BIG, INT_BIG);
+                wrote = true;
+            }
+            __syncwarp();
+            const int amin = col[ia], amax = col[n - 1];
+            if (nb <= amax) {
+                if (pos < 0) pos = r_a <= 0 ? 0 : lower_bound_from(B, sl.pdeg, 0, amin, lane);
+                nb = chunk_members(B, sl.pdeg, pos, amin, amax, ia, n, area, lane);
+                some = true;
+            }
+            if (prev >= amin && prev <= amax) {
+                uint32_t a[1] = {smem_u32(col)};
+                const int x[1] = {prev};
+                lb_search(a, x, n);
+                if (lds_at<0>(a[0]) == prev) prevpos = (int)(a[0] - smem_u32(col)) >> 2;
+            }
+            if (wrote) fence_proxy_async_cta();  // the columns are overwritten by the next copy
+            __syncwarp();
+            if (lane == 0 && r0 + CHUNK < lim) {
+                const int rn = r0 + CHUNK, k = min(min(CHUNK, (lim - rn + 15) & ~15), whole - rn);
+                mbar_arrive_expect_tx(bar, (uint32_t)max(k, 0) * 4u);
+                if (k > 0) tma_load_1d(col, g.col + beg + rn, (uint32_t)k * 4u, bar);
+            }
+        }
+#pragma unroll 1
+        for (int rp = r0; rp < min(lim, r0 + (N2V ? CHUNK : PAIR)); rp += PAIR) {
+            float w[16];
+            load_pair<LAB>(wrow, lrow, want, rp, lim, left, lane, w);
+            if (n2v) {
+                const float f1 = sl.rq.fac_f[1], f2 = sl.rq.fac_f[2];
+                unsigned mk[4] = {0u, 0u, 0u, 0u};
+                if (some) {
+                    const unsigned* mw = reinterpret_cast<const unsigned*>(area + Area<N2V>::MASK + (rp - r0)) + lane;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) mk[k] = mw[32 * k];
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    w[j] = __fmul_rn(w[j], mk[j >> 2] >> (8 * (j & 3)) & 1u ? f1 : f2);
+                const int pp = prevpos - (rp - r0);
+                if (prevpos >= 0 && (unsigned)pp < (unsigned)PAIR) {
+                    // the return factor in place of the other two
+                    const float wp = __fmul_rn(__ldg(wrow + rp + pp), sl.rq.fac_f[0]);
+                    const int jp = (pp >> 2 & 31) == lane ? (pp >> 7) * 4 + (pp & 3) : -1;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (j == jp) w[j] = wp;
+                }
+            }
+            offer_pair(R, w, rp + STAGE < lim, rp, lane, sl, stream);
+        }
+        if (N2V) __syncwarp();  // the membership bytes are cleared for the next chunk
+    }
+    return true;
 }
 
 __device__ __forceinline__ int find_req(const ReqDev* __restrict__ reqs, int n_req, long long gq) {
@@ -405,17 +684,20 @@ __device__ __forceinline__ void fetch_row(const GraphDev& g, Slot& s, int v) {
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Commit a move of slot s (one thread): append `next` to the path, advance
-// the walk, apply the PPR stop test and the length limit, fetch the next
-// row's offsets, and hand the slot back (READY or FINISH).  `hub`: the slot
-// may belong to another warp, so the offsets must have landed first.
-__device__ __forceinline__ void commit(const GraphDev& g, Slot& s, long long beg, int d, int sel, uint64_t seed,
-                                       uint64_t qid, uint32_t t, bool hub) {
+// Commit a move of slot s (one thread): append the entry at row index `sel` to
+// the path, advance the walk, apply the PPR stop test and the length limit,
+// fetch the next row's offsets, and hand the slot back (READY or FINISH).
+// `hub`: the slot may belong to another warp, so the offsets must have landed
+// first.
+__device__ __forceinline__ void commit(const GraphDev& g, Slot& s, int sel, bool hub) {
     const ReqDev& R = s.rq;
+    const long long beg = s.row[0];
+    const int d = (int)(s.row[1] - beg);
     const int next = __ldg(g.col + beg + sel);
     fetch_row(g, s, next);
+    const int t = s.t;
     bool stop = false;
-    if (R.algo == FW_PPR) stop = step_block(seed, qid, t).z < R.t_stop;
+    if (R.algo == FW_PPR) stop = step_block(R.seed, (uint64_t)(R.q_id0 + s.q), (uint32_t)t).z < R.t_stop;
     const int k = s.k;
     R.paths[s.q * ((long long)R.max_len + 1) + k] = next;
     s.k = k + 1;
@@ -423,8 +705,8 @@ __device__ __forceinline__ void commit(const GraphDev& g, Slot& s, long long beg
     s.pbeg = beg;
     s.pdeg = d;
     s.cur = next;
-    s.t = (int)t + 1;
-    stop = stop || (int)t + 1 >= s.lim;
+    s.t = t + 1;
+    stop = stop || t + 1 >= s.lim;
     if (hub) {
         cp_async_wait_all();
         __threadfence_block();
@@ -432,13 +714,12 @@ __device__ __forceinline__ void commit(const GraphDev& g, Slot& s, long long beg
     *(volatile int*)&s.state = stop ? ST_FINISH : ST_READY;
 }
 
-// Claim one segment of an open hub task: (h, j) = task, segment; false if
-// none is open.  Warp-collective, uniform result.
-__device__ __forceinline__ bool hub_claim(CtaHead& H0, int lane, int& h, int& j) {
-    h = -1;
-    j = -1;
-    if (!__shfl_sync(FULL, *(volatile int*)&H0.hub_open, 0)) return false;
+// Claim one segment of an open hub task: task << 8 | segment, or -1 if none is
+// open.  Warp-collective, uniform result.
+__device__ __noinline__ int hub_claim(CtaHead& H0, int lane) {
+    int got = -1;
     if (lane == 0) {
+#pragma unroll 1
         for (int i = 0; i < NHUB; ++i) {
             HubTask& H = H0.hub[i];
             const unsigned v = *(volatile unsigned*)&H.ctl;
@@ -447,36 +728,262 @@ __device__ __forceinline__ bool hub_claim(CtaHead& H0, int lane, int& h, int& j)
             // a claim counts only if the task was live then; the task cannot
             // be freed before this segment is done, so its fields stay valid
             if ((old & H_STATE) == H_ACTIVE && hub_next(old) < hub_nseg(old)) {
-                h = i;
-                j = hub_next(old);
-                if (j == hub_nseg(old) - 1) atomicSub(&H0.hub_open, 1);
+                got = i << 8 | hub_next(old);
+                if (hub_next(old) == hub_nseg(old) - 1) atomicSub(&H0.hub_open, 1);
+                break;
+            }
+        }
+        __threadfence_block();
+    }
+    return __shfl_sync(FULL, got, 0);
+}
+
+// What the engine's out-of-line parts share.
+struct Launch {
+    const ReqDev* reqs;  // null: the table inside the parameter block
+    int n_req;
+    long long total;
+    unsigned long long* cursor;
+    unsigned long long* counters;
+};
+
+// Claim one query for the empty slot sl: the slot's new state, ST_EMPTY if
+// nothing is published right now (served form), -1 if no query is left.
+// Out of line (once per walk, and it keeps the step loop's code small).
+// Warp-collective, uniform result.
+template <bool N2V, bool SERVE>
+__device__ __noinline__ int claim_query(const GraphDev& g, const ReqDev* __restrict__ reqs, const Launch& L, const ServeDev& sv,
+                                        Slot& sl, int lane) {
+    // lane 0: r = the query's request, qi = its index inside the request
+    long long qi = -1;
+    int r = 0;
+    if (SERVE) {
+        // the oldest published request with queries left hands out its next
+        // one; once the host asks the engine to stop, nothing new is claimed
+        if (lane == 0 && !*sv.stop) {
+#pragma unroll 1
+            for (int tries = 0; tries < 64; ++tries) {
+                const unsigned long long hd = *(volatile unsigned long long*)sv.head;
+                if ((long long)hd >= *sv.pub_r) break;
+                const int rs = (int)(hd % (unsigned long long)sv.maxr);
+                const unsigned long long old = atomicAdd(&sv.taken[rs], 1ull);
+                if (old < kTakenBase) {
+                    qi = (long long)(old + (unsigned long long)__ldcg(&sv.ring[rs].n_q) - kTakenBase);
+                    r = rs;
+                    break;
+                }
+                atomicCAS(sv.head, hd, hd + 1);  // exhausted: move the head on
+            }
+        }
+        qi = __shfl_sync(FULL, qi, 0);
+        if (qi < 0) return ST_EMPTY;
+    } else {
+        long long gq = 0;
+        if (lane == 0) gq = (long long)atomicAdd(L.cursor, 1ull);
+        gq = __shfl_sync(FULL, gq, 0);
+        if (gq >= L.total) return -1;
+        r = find_req(reqs, L.n_req, gq);
+        qi = gq - reqs[r].q_begin;
+    }
+    // the walk's own copy of its request (through L2: a served ring slot is
+    // rewritten between requests)
+    r = __shfl_sync(FULL, r, 0);
+    constexpr int RW = (int)(sizeof(ReqDev) / 8);
+    static_assert(sizeof(ReqDev) % 8 == 0 && RW <= 32, "request copy: one word per lane");
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&reqs[r]);
+    if (lane < RW) reinterpret_cast<unsigned long long*>(&sl.rq)[lane] = SERVE ? __ldcg(src + lane) : src[lane];
+    __syncwarp();
+    int st = 0;
+    if (lane == 0) {
+        const ReqDev& Rq = sl.rq;
+        const int start = __ldcg(Rq.starts + qi);
+        const int pv = Rq.prev ? __ldcg(Rq.prev + qi) : -1;
+        const int t0 = Rq.step0 ? __ldcg(Rq.step0 + qi) : 0;
+        const int lim = Rq.lengths ? __ldcg(Rq.lengths + qi) : Rq.max_len;
+        sl.q = qi;
+        sl.req = r;
+        sl.k = 0;
+        if (start < 0 || start >= g.n || pv < -1 || pv >= g.n || t0 < 0) {
+            atomicAdd(&L.counters[C_BAD_INPUT], 1ull);
+            st = ST_FINISH;  // written out as an empty path
+        } else {
+            fetch_row(g, sl, start);
+            Rq.paths[qi * ((long long)Rq.max_len + 1)] = start;
+            sl.k = 1;
+            sl.cur = start;
+            sl.prev = pv;
+            sl.t = t0;
+            sl.lim = min(lim, Rq.max_len);
+            sl.pbeg = 0;
+            sl.pdeg = 0;
+            if (N2V && pv >= 0) {
+                const long long pb = __ldg(g.row_ptr + pv);
+                sl.pbeg = pb;
+                sl.pdeg = (int)(__ldg(g.row_ptr + pv + 1) - pb);
+            }
+            st = t0 >= sl.lim ? ST_FINISH : ST_READY;
+        }
+        sl.state = st;
+    }
+    st = __shfl_sync(FULL, st, 0);
+    __syncwarp();
+    return st;
+}
+
+// Retire a finished walk: path_len and -1 padding; the slot is empty then.
+// Warp-collective.
+template <bool SERVE>
+__device__ __noinline__ void retire_walk(const ServeDev& sv, Slot& sl, unsigned long long* cnt, int lane) {
+    const ReqDev& Rq = sl.rq;
+    const long long width = (long long)Rq.max_len + 1;
+    const int k = sl.k;
+    int32_t* row = Rq.paths + sl.q * width;
+#pragma unroll 1
+    for (long long e = k + lane; e < width; e += 32) row[e] = -1;
+    if (lane == 0) {
+        Rq.path_len[sl.q] = k;
+        cnt[N_WALKS] += 1;
+        sl.state = ST_EMPTY;
+        if (SERVE) {
+            // the request's last walk tells the host (all its writes are
+            // visible first)
+            __threadfence();
+            const int rs = sl.req;
+            if (atomicAdd(&sv.done[rs], 1ull) + 1 == (unsigned long long)Rq.n_q) {
+                __threadfence_system();
+                sv.complete[rs] = global_timer_ns() | 1ull;
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// Publish the step of slot sl as a CTA hub task of nseg segments, if a task
+// entry is free; if none is, the walk stays ready and is published on a later
+// visit, after this warp has helped the open tasks.  Warp-collective.
+__device__ __noinline__ void hub_publish(CtaHead& head, WarpHead& wh, Slot& sl, int slot, int nseg, int lane) {
+    int ok = 0;
+    if (lane == 0) {
+#pragma unroll 1
+        for (int i = 0; i < NHUB; ++i) {
+            HubTask& H = head.hub[i];
+            const unsigned vv = *(volatile unsigned*)&H.ctl;
+            if ((vv & H_STATE) == H_FREE && atomicCAS(&H.ctl, vv, H_SETUP) == vv) {
+                H.slot = slot;
+                H.done_seg = 0;
+                H.best = ~0ull;
+                sl.state = ST_HUB;
+                __threadfence_block();
+                atomicExch(&H.ctl, H_ACTIVE | (unsigned)nseg << 16);
+                atomicAdd(&head.hub_open, 1);
+                ok = 1;
                 break;
             }
         }
     }
-    h = __shfl_sync(FULL, h, 0);
-    j = __shfl_sync(FULL, j, 0);
-    if (h >= 0) __threadfence_block();
-    return h >= 0;
+    if (!__shfl_sync(FULL, ok, 0)) {
+        const unsigned nap = wh.nap;
+        __nanosleep(nap);
+        __syncwarp();
+        if (lane == 0) wh.nap = min(nap * 2u, 1024u);
+        __syncwarp();
+    }
 }
 
+// The walk to advance when the next one in turn is not ready: refills empty
+// slots, retires finished walks, waits when there is nothing to do.  A slot
+// index, PICK_AGAIN (look for hub work first), or PICK_QUIT.  Out of line: a
+// call per few steps.  Warp-collective, uniform result.
+enum { PICK_QUIT = -1, PICK_AGAIN = -2 };
+template <bool N2V, bool SERVE>
+__device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restrict__ reqs, const Launch& L,
+                                      const ServeDev& sv, CtaHead& head, WarpHead& wh, Slot* mine, int sw, int rr,
+                                      int lane) {
+    bool waiting = false;
+#pragma unroll 1
+    for (int i = 0; i < sw; ++i) {
+        int jj = rr + i;
+        if (jj >= sw) jj -= sw;
+        Slot& sl = mine[jj];
+        // another warp may flip a hub-parked slot at any time: let lane 0
+        // read it once for the whole warp
+        int st = __shfl_sync(FULL, *(volatile int*)&sl.state, 0);
+        if (st == ST_EMPTY && !wh.exhausted) {
+            st = claim_query<N2V, SERVE>(g, reqs, L, sv, sl, lane);
+            if (st < 0) {
+                if (lane == 0) wh.exhausted = 1;
+                __syncwarp();
+            }
+        }
+        if (st == ST_FINISH) {
+            retire_walk<SERVE>(sv, sl, wh.cnt, lane);
+            --i;  // revisit this slot: it can be refilled now
+            continue;
+        }
+        if (st == ST_HUB) waiting = true;
+        if (st == ST_READY) return jj;
+    }
+    // Nothing to do now.  Batch: done once every slot is empty.  Served: poll
+    // for new requests; return once the host asks to stop.  Either way a wait
+    // lasts 2 s at most.
+    if (!waiting && !SERVE) return PICK_QUIT;
+    int quit = 0;
+    if (lane == 0) {
+        const unsigned long long now = global_timer_ns();
+        if (wh.idle_since == 0) wh.idle_since = now;
+        const bool late = now - wh.idle_since > kWaitLimitNs;
+        if (!waiting) {
+            quit = late || *sv.stop;
+        } else {
+            if (late) {
+                atomicAdd(&L.counters[C_TIMEOUT], 1ull);
+                head.abort_flag = 1;
+            }
+            quit = *(volatile int*)&head.abort_flag;
+        }
+    }
+    if (__shfl_sync(FULL, quit, 0)) return PICK_QUIT;
+    // back off: an idle warp's polling takes issue slots from the warps that
+    // are scanning
+    const unsigned nap = wh.nap;
+    __nanosleep(nap);
+    __syncwarp();
+    if (lane == 0) wh.nap = min(nap * 2u, waiting ? 1024u : 32768u);
+    __syncwarp();
+    return PICK_AGAIN;
+}
+
+// N2V, LAB: the launch may hold node2vec / MetaPath requests (a build without
+// them is smaller: see the instruction cache above).
 // SERVE: the served form's build (queries claimed from the request ring,
 // completion stamps, idle polling); the batch build compiles all of that out.
-template <bool N2V, bool SERVE>
-__global__ void __launch_bounds__(512, N2V ? 1 : 2)
-    fast_kernel(GraphDev g, const __grid_constant__ ReqTable tab, int n_req, long long total, unsigned long long* cursor,
-                unsigned long long* counters, int sw, int d_t, ServeDev sv) {
-    const ReqDev* __restrict__ reqs = SERVE ? sv.ring : (tab.ext ? tab.ext : tab.r);
+template <bool N2V, bool LAB, bool SERVE>
+// Registers: 64 a thread for first-order launches (32 warps per SM), 80 for
+// node2vec (24 warps; 128 registers and 16 warps measured 241 ms against 202
+// on the R-MAT-25 batch of 2^18 walks, 64 registers with spills 248).
+__global__ void __maxnreg__(N2V ? 80 : 64)
+    fast_kernel(const __grid_constant__ GraphDev g, const __grid_constant__ ReqTable tab, const __grid_constant__ Launch L,
+                int sw, int d_t, const __grid_constant__ ServeDev sv) {
+    const ReqDev* __restrict__ reqs = SERVE ? sv.ring : (L.reqs ? L.reqs : tab.r);
     extern __shared__ __align__(128) unsigned char dyn[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     CtaHead& head = *reinterpret_cast<CtaHead*>(dyn);
     unsigned char* area = dyn + kHeadBytes + warp * Area<N2V>::BYTES;
     Slot* slots = reinterpret_cast<Slot*>(dyn + kHeadBytes + nwarp * Area<N2V>::BYTES);
-    Slot* mine = slots + warp * sw;
     WarpHead& wh = *reinterpret_cast<WarpHead*>(area + Area<N2V>::HEAD);
-    unsigned long long* cnt = wh.cnt;
-    if (lane < N_COUNTS) cnt[lane] = 0;
-    if (lane < sw) mine[lane].state = ST_EMPTY;
+    uint32_t ph = 0;  // parity at which the next chunk's columns land
+    if (N2V && lane == 0) {
+        mbar_init(reinterpret_cast<unsigned long long*>(area + Area<N2V>::BAR), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        reinterpret_cast<int*>(area + Area<N2V>::COL)[CHUNK] = INT_MIN;
+    }
+    if (lane < N_COUNTS) wh.cnt[lane] = 0;
+    if (lane < sw) slots[warp * sw + lane].state = ST_EMPTY;
+    if (lane == 0) {
+        wh.idle_since = 0;
+        wh.nap = 128;
+        wh.exhausted = 0;
+    }
     if (threadIdx.x < NHUB) head.hub[threadIdx.x].ctl = H_FREE;
     if (threadIdx.x == 0) {
         head.hub_open = 0;
@@ -484,248 +991,46 @@ __global__ void __launch_bounds__(512, N2V ? 1 : 2)
     }
     __syncthreads();
 
-    bool exhausted = false;
     int rr = 0;
-    unsigned long long idle_since = 0;
-    unsigned nap = 128;  // idle back-off (ns)
-
+#pragma unroll 1
     for (;;) {
         // ------------------------------------------------ choose the work
         // Either one segment of an open hub task (their owners are waiting,
         // so they come first) or one step of one of this warp's own walks.
-        StepCtx c;
-        Stream S;
-        int ra, lim, sq;  // row indices [ra, lim) to scan, sq at a time
-        int h, j, s = -1;
-        const bool seg = hub_claim(head, lane, h, j);
-        if (seg) {
-            const HubTask& H = head.hub[h];
-            c = H.c;
-            sq = H.seg_e;
-            ra = -(int)(c.beg & 15) + j * sq;
-            lim = min(c.d, ra + sq);
-            S.seed = H.seed;
-            S.qid = H.qid;
-            S.t = H.t;
-            S.id = (uint32_t)j;
+        int seg = -1, s;
+        if (__shfl_sync(FULL, *(volatile int*)&head.hub_open, 0)) seg = hub_claim(head, lane);
+        if (seg >= 0) {
+            s = head.hub[seg >> 8].slot;
         } else {
-            // ---- pick a walk: refill empty slots, retire finished ones ----
-            bool waiting = false;
-            for (int i = 0; i < sw; ++i) {
-                int jj = rr + i;
-                if (jj >= sw) jj -= sw;
-                Slot& sl = mine[jj];
-                // another warp may flip a hub-parked slot at any time: let
-                // lane 0 read it once for the whole warp
-                int st = __shfl_sync(FULL, *(volatile int*)&sl.state, 0);
-                if (st == ST_EMPTY && !exhausted) {
-                    // claim one query (lane 0): r = its request, qi = its
-                    // index inside the request; -1 if none
-                    long long qi = -1;
-                    int r = 0;
-                    if (SERVE) {
-                        // the oldest published request with queries left
-                        // hands out its next one; once the host asks the
-                        // engine to stop, nothing new is claimed
-                        if (lane == 0 && !*sv.stop) {
-                            for (int tries = 0; tries < 64; ++tries) {
-                                const unsigned long long hd = *(volatile unsigned long long*)sv.head;
-                                if ((long long)hd >= *sv.pub_r) break;
-                                const int rs = (int)(hd % (unsigned long long)sv.maxr);
-                                const unsigned long long old = atomicAdd(&sv.taken[rs], 1ull);
-                                if (old < kTakenBase) {
-                                    qi = (long long)(old + (unsigned long long)__ldcg(&sv.ring[rs].n_q) - kTakenBase);
-                                    r = rs;
-                                    break;
-                                }
-                                atomicCAS(sv.head, hd, hd + 1);  // exhausted: move the head on
-                            }
-                        }
-                        qi = __shfl_sync(FULL, qi, 0);
-                        if (qi < 0) continue;  // nothing published right now: the slot stays empty
-                    } else {
-                        long long gq = 0;
-                        if (lane == 0) gq = (long long)atomicAdd(cursor, 1ull);
-                        gq = __shfl_sync(FULL, gq, 0);
-                        if (gq >= total) {
-                            exhausted = true;
-                            continue;
-                        }
-                        r = find_req(reqs, n_req, gq);
-                        qi = gq - reqs[r].q_begin;
-                    }
-                    // the walk's own copy of its request (through L2: a
-                    // served ring slot is rewritten between requests)
-                    r = __shfl_sync(FULL, r, 0);
-                    constexpr int RW = (int)(sizeof(ReqDev) / 8);
-                    static_assert(sizeof(ReqDev) % 8 == 0 && RW <= 32, "request copy: one word per lane");
-                    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&reqs[r]);
-                    if (lane < RW)
-                        reinterpret_cast<unsigned long long*>(&sl.rq)[lane] = SERVE ? __ldcg(src + lane) : src[lane];
-                    __syncwarp();
-                    if (lane == 0) {
-                        const ReqDev& Rq = sl.rq;
-                        const int start = __ldcg(Rq.starts + qi);
-                        const int pv = Rq.prev ? __ldcg(Rq.prev + qi) : -1;
-                        const int t0 = Rq.step0 ? __ldcg(Rq.step0 + qi) : 0;
-                        const int lim = Rq.lengths ? __ldcg(Rq.lengths + qi) : Rq.max_len;
-                        sl.q = qi;
-                        sl.req = r;
-                        sl.k = 0;
-                        if (start < 0 || start >= g.n || pv < -1 || pv >= g.n || t0 < 0) {
-                            atomicAdd(&counters[C_BAD_INPUT], 1ull);
-                            st = ST_FINISH;  // written out as an empty path
-                        } else {
-                            fetch_row(g, sl, start);
-                            Rq.paths[qi * ((long long)Rq.max_len + 1)] = start;
-                            sl.k = 1;
-                            sl.cur = start;
-                            sl.prev = pv;
-                            sl.t = t0;
-                            sl.lim = min(lim, Rq.max_len);
-                            sl.pbeg = 0;
-                            sl.pdeg = 0;
-                            if (N2V && pv >= 0) {
-                                const long long pb = __ldg(g.row_ptr + pv);
-                                sl.pbeg = pb;
-                                sl.pdeg = (int)(__ldg(g.row_ptr + pv + 1) - pb);
-                            }
-                            st = t0 >= sl.lim ? ST_FINISH : ST_READY;
-                        }
-                        sl.state = st;
-                    }
-                    st = __shfl_sync(FULL, st, 0);
-                    __syncwarp();
-                }
-                if (st == ST_FINISH) {
-                    // retire: path_len and -1 padding
-                    const ReqDev& Rq = sl.rq;
-                    const long long width = (long long)Rq.max_len + 1;
-                    const int k = sl.k;
-                    int32_t* row = Rq.paths + sl.q * width;
-                    for (long long e = k + lane; e < width; e += 32) row[e] = -1;
-                    if (lane == 0) {
-                        Rq.path_len[sl.q] = k;
-                        cnt[N_WALKS] += 1;
-                        sl.state = ST_EMPTY;
-                        if (SERVE) {
-                            // the request's last walk tells the host (all its
-                            // writes are visible first)
-                            __threadfence();
-                            const int rs = sl.req;
-                            if (atomicAdd(&sv.done[rs], 1ull) + 1 == (unsigned long long)Rq.n_q) {
-                                __threadfence_system();
-                                sv.complete[rs] = global_timer_ns() | 1ull;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    --i;  // revisit this slot: it can be refilled now
-                    continue;
-                }
-                if (st == ST_HUB) waiting = true;
-                if (st == ST_READY) {
-                    s = jj;
-                    rr = jj + 1 == sw ? 0 : jj + 1;
-                    break;
-                }
+            s = rr;
+            if (__shfl_sync(FULL, *(volatile int*)&slots[warp * sw + rr].state, 0) != ST_READY) {
+                s = pick_walk<N2V, SERVE>(g, reqs, L, sv, head, wh, slots + warp * sw, sw, rr, lane);
+                if (s == PICK_QUIT) break;
+                if (s < 0) continue;
             }
-            if (s < 0) {
-                // nothing to do now.  Batch: done once every slot is empty.
-                // Served: poll for new requests; return once the host asks
-                // to stop.  Either way a wait lasts 2 s at most.
-                if (!waiting && !SERVE) break;
-                int quit = 0;
-                if (lane == 0) {
-                    const unsigned long long now = global_timer_ns();
-                    if (idle_since == 0) idle_since = now;
-                    const bool late = now - idle_since > kWaitLimitNs;
-                    if (!waiting) {
-                        quit = late || *sv.stop;
-                    } else {
-                        if (late) {
-                            atomicAdd(&counters[C_TIMEOUT], 1ull);
-                            head.abort_flag = 1;
-                        }
-                        quit = *(volatile int*)&head.abort_flag;
-                    }
-                }
-                if (__shfl_sync(FULL, quit, 0)) break;
-                // back off: an idle warp's polling takes issue slots from the
-                // warps that are scanning
-                __nanosleep(nap);
-                nap = min(nap * 2u, waiting ? 1024u : 32768u);
-                continue;
-            }
-
-            // ---- one step of slot s ----
-            Slot& sl = mine[s];
-            if (lane == 0) cp_async_wait_all();
+            rr = s + 1 == sw ? 0 : s + 1;
+            s += warp * sw;
+            if (lane == 0) cp_async_wait_all();  // the offsets of its row
             __syncwarp();
-            const long long beg = sl.row[0];
-            const int d = (int)(sl.row[1] - beg);
-            if (d == 0) {  // dead end
-                if (lane == 0) sl.state = ST_FINISH;
-                __syncwarp();
-                continue;
-            }
-            S.t = (uint32_t)sl.t;
-            c.beg = beg;
-            c.d = d;
-            c.algo = sl.rq.algo;
-            c.want = c.algo == FW_METAPATH ? (int)sl.rq.schema[S.t % (uint32_t)sl.rq.schema_len] : -1;
-            if (N2V) {
-                c.pbeg = sl.pbeg;
-                c.pdeg = sl.pdeg;
-                c.prev = sl.prev;
-                c.f0 = sl.rq.fac_f[0];
-                c.f1 = sl.rq.fac_f[1];
-                c.f2 = sl.rq.fac_f[2];
-            }
-            S.qid = (uint64_t)(sl.rq.q_id0 + sl.q);
-            S.seed = sl.rq.seed;
-            S.id = 0;
-            ra = -(int)(beg & 15);  // the scan starts on a 16-entry group
-            lim = d;
-            sq = seg_entries(ra, d);
-
-            if (d > d_t) {
-                // publish as a CTA hub task, if a task entry is free
-                int ok = 0;
-                if (lane == 0) {
-                    for (int i = 0; i < NHUB; ++i) {
-                        HubTask& H = head.hub[i];
-                        const unsigned vv = *(volatile unsigned*)&H.ctl;
-                        if ((vv & H_STATE) == H_FREE && atomicCAS(&H.ctl, vv, H_SETUP) == vv) {
-                            H.slot = (int)(&sl - slots);
-                            H.seg_e = sq;
-                            H.done_seg = 0;
-                            H.best = ~0ull;
-                            H.c = c;
-                            H.seed = S.seed;
-                            H.qid = S.qid;
-                            H.t = S.t;
-                            sl.state = ST_HUB;
-                            __threadfence_block();
-                            atomicExch(&H.ctl, H_ACTIVE | (unsigned)((d - ra + sq - 1) / sq) << 16);
-                            atomicAdd(&head.hub_open, 1);
-                            ok = 1;
-                            break;
-                        }
-                    }
-                }
-                if (!__shfl_sync(FULL, ok, 0)) {
-                    // no free task entry: the walk stays ready and is
-                    // published on a later visit, after this warp has helped
-                    // the open tasks
-                    __nanosleep(nap);
-                    nap = min(nap * 2u, 1024u);
-                }
-                continue;
-            }
         }
-        idle_since = 0;
-        nap = 128;
+        Slot& sl = slots[s];
+        int lim = (int)(sl.row[1] - sl.row[0]);
+        int ra = lim ? -(int)(sl.row[0] & 15) : 0;  // the scan starts on a 16-entry group (a dead end has none)
+        int stream = 0;
+        const int sq = seg_entries(ra, lim);
+        if (seg >= 0) {
+            stream = seg & 0xFF;
+            ra += stream * sq;
+            lim = min(lim, ra + sq);
+        } else if (lim > d_t) {
+            hub_publish(head, wh, sl, s, (lim - ra + sq - 1) / sq, lane);
+            continue;
+        }
+
+        if (lane == 0) {
+            wh.idle_since = 0;
+            wh.nap = 128;
+        }
 
         // ------------------------------------ stream the row range (one site)
         // A hub segment is one range.  A row sampled by this warp alone is
@@ -733,40 +1038,47 @@ __global__ void __launch_bounds__(512, N2V ? 1 : 2)
         // stream j, and the step keeps the smallest (race time, index) over
         // them, as a hub task's merge does.
         unsigned long long best = ~0ull;
+        bool scanned = true;
+#pragma unroll 1
         for (; ra < lim; ra += sq) {
             Res R;
             R.init();
-            scan_range<N2V>(g, c, ra, min(lim, ra + sq), lane, R, S);
+            if (!scan_range<N2V, LAB>(g, sl, ra, min(lim, ra + sq), lane, area, ph, R, stream)) {
+                scanned = false;
+                break;
+            }
             if (R.sel >= 0) best = min(best, race_key(R));
-            ++S.id;
+            ++stream;
+        }
+        if (N2V && !scanned) {
+            if (lane == 0) atomicAdd(&L.counters[C_TIMEOUT], 1ull);
+            break;
         }
 
         // ------------------------------------------------ use the result
         if (lane == 0) {
-            Slot* sp = &mine[max(s, 0)];
             bool fin = true;
-            if (seg) {
+            if (seg >= 0) {
                 // fold the segment into its hub task; the warp that completes
                 // the last segment finishes the step
-                HubTask& H = head.hub[h];
+                HubTask& H = head.hub[seg >> 8];
                 if (best != ~0ull) atomicMin(&H.best, best);
                 __threadfence_block();
                 fin = atomicAdd(&H.done_seg, 1) == hub_nseg(*(volatile unsigned*)&H.ctl) - 1;
                 __threadfence_block();
-                sp = &slots[H.slot];
                 best = *(volatile unsigned long long*)&H.best;
             }
             if (fin) {
                 if (best == ~0ull) {
                     __threadfence_block();
-                    *(volatile int*)&sp->state = ST_FINISH;  // nothing selectable: the walk stops here
+                    *(volatile int*)&sl.state = ST_FINISH;  // nothing selectable: the walk stops here
                 } else {
-                    count_step(cnt, c.d, c.algo, seg);
-                    commit(g, *sp, c.beg, c.d, (int)(best & 0xFFFFFFFFull), S.seed, S.qid, S.t, seg);
+                    count_step(wh.cnt, (int)(sl.row[1] - sl.row[0]), sl.rq.algo, seg >= 0);
+                    commit(g, sl, (int)(best & 0xFFFFFFFFull), seg >= 0);
                 }
-                if (seg) {
+                if (seg >= 0) {
                     __threadfence_block();
-                    atomicExch(&head.hub[h].ctl, H_FREE);
+                    atomicExch(&head.hub[seg >> 8].ctl, H_FREE);
                 }
             }
         }
@@ -774,7 +1086,7 @@ __global__ void __launch_bounds__(512, N2V ? 1 : 2)
     }
     cp_async_wait_all();
     __syncwarp();
-    if (lane == 0) flush_counts(cnt, counters);
+    if (lane == 0) flush_counts(wh.cnt, L.counters);
 }
 
 }  // namespace

@@ -24,22 +24,38 @@ cudaError_t engine_grid(K kern, int threads, size_t smem, const Tuning& tu, int*
 
 }  // namespace
 
-cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
-                        unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
-    auto kern = fast_kernel<false, false>;
-    const int warps = tu.block_threads / 32;
-    const int sw = max(1, min(SW_MAX, tu.slots / warps));
-    const size_t smem = cta_smem<false>(warps, sw);
+template <bool N2V, bool LAB>
+static cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                      unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
+    auto kern = fast_kernel<N2V, LAB, false>;
+    const int sw = max(1, min(SW_MAX, tu.slots / (tu.block_threads / 32)));
+    // CTAs of 256 threads unless the caller chose: at 80 registers three of
+    // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
+    // (R-MAT-25 node2vec: 240 -> 202 ms), and a hub row's last segments hold
+    // back 8 warps instead of 16 (PPR from the R-MAT-22 hub: 5.7 -> 4.8 ms).
+    const int threads = tu.own_shape || tu.ctas_per_sm > 0 ? tu.block_threads : 256;
+    const int warps = threads / 32;
+    const size_t smem = cta_smem<N2V>(warps, sw);
     int sms = 0, per_sm = 0;
-    cudaError_t e = engine_grid(kern, tu.block_threads, smem, tu, &sms, &per_sm);
+    cudaError_t e = engine_grid(kern, threads, smem, tu, &sms, &per_sm);
     if (e != cudaSuccess) return e;
     const int64_t per_cta = (int64_t)sw * warps;
     const int64_t grid = min((int64_t)sms * per_sm, (total + per_cta - 1) / per_cta);
     ServeDev none;
     memset(&none, 0, sizeof none);
-    kern<<<(unsigned)grid, tu.block_threads, smem, stream>>>(g, reqs, n_req, (long long)total, cursor, counters, sw,
-                                                             tu.d_warp, none);
+    // (a table inside the parameter block is found by the kernel itself)
+    const Launch L = {reqs.ext, n_req, (long long)total, cursor, counters};
+    kern<<<(unsigned)grid, threads, smem, stream>>>(g, reqs, L, sw, tu.d_warp, none);
     return cudaGetLastError();
+}
+
+cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                        unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
+    const bool n2v = reqs.algos >> FW_NODE2VEC & 1u, lab = reqs.algos >> FW_METAPATH & 1u;
+    return n2v ? (lab ? launch_as<true, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
+                      : launch_as<true, false>(g, reqs, n_req, total, cursor, counters, tu, stream))
+               : (lab ? launch_as<false, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
+                      : launch_as<false, false>(g, reqs, n_req, total, cursor, counters, tu, stream));
 }
 
 }  // namespace fw

@@ -148,6 +148,7 @@ struct Tuning {
     int slots;
     int d_warp;
     int ctas_per_sm;
+    bool own_shape;  // block_threads was set by the caller (else each engine may take the CTA size that suits it)
 };
 
 // Launch the persistent walk engine over `n_req` requests (device array

@@ -1830,11 +1830,14 @@ cudaError_t launch_serve_one(const GraphDev& g, const ServeDev& sv, Scratch* scr
 
 }  // namespace
 
-Tuning default_tuning() { return Tuning{512, 64, 65536, 0}; }
+Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false}; }
 
 Tuning sanitize_tuning(Tuning t) {
     const Tuning d = default_tuning();
-    if (t.block_threads != 128 && t.block_threads != 256 && t.block_threads != 512) t.block_threads = d.block_threads;
+    if (t.block_threads != 128 && t.block_threads != 256 && t.block_threads != 512) {
+        t.block_threads = d.block_threads;
+        t.own_shape = false;
+    }
     if (t.slots <= 0) t.slots = 4 * (t.block_threads / 32);  // four walks per warp
     if (t.slots > (t.block_threads / 32) * SW_MAX) t.slots = (t.block_threads / 32) * SW_MAX;
     if (t.d_warp <= 0) t.d_warp = d.d_warp;
@@ -1867,18 +1870,14 @@ cudaError_t launch_walk(const GraphDev& g, int mode, const ReqTable& reqs, int n
     const Tuning tu = sanitize_tuning(tune);
     if (total <= 0) return cudaSuccess;
     const bool exact = mode == FW_EXACT;
-    if (!exact && !(reqs.algos >> FW_NODE2VEC & 1u))
-        return launch_fast(g, reqs, n_req, total, cursor, counters, tu, stream);
+    if (!exact) return launch_fast(g, reqs, n_req, total, cursor, counters, tu, stream);
     switch (tu.block_threads) {
         case 128:
-            return exact ? launch_one<MODE_EXACT, 128>(g, reqs, n_req, total, cursor, counters, tu, stream)
-                         : launch_one<MODE_FAST, 128>(g, reqs, n_req, total, cursor, counters, tu, stream);
+            return launch_one<MODE_EXACT, 128>(g, reqs, n_req, total, cursor, counters, tu, stream);
         case 512:
-            return exact ? launch_one<MODE_EXACT, 512>(g, reqs, n_req, total, cursor, counters, tu, stream)
-                         : launch_one<MODE_FAST, 512>(g, reqs, n_req, total, cursor, counters, tu, stream);
+            return launch_one<MODE_EXACT, 512>(g, reqs, n_req, total, cursor, counters, tu, stream);
         default:
-            return exact ? launch_one<MODE_EXACT, 256>(g, reqs, n_req, total, cursor, counters, tu, stream)
-                         : launch_one<MODE_FAST, 256>(g, reqs, n_req, total, cursor, counters, tu, stream);
+            return launch_one<MODE_EXACT, 256>(g, reqs, n_req, total, cursor, counters, tu, stream);
     }
 }
 

@@ -71,3 +71,38 @@ def test_fast_laws_at_tile_edges(algo, d_warp):
         assert (at < d).all() and (g.col[row][at] == nxt[i]).all(), (algo, d)
         _, p = chi2_tv(np.bincount(at, minlength=d), w / w.sum(), N)
         assert p > P_MIN, (algo, d, p)
+
+
+# node2vec: rows of prev that make every kind of window: none, a few values, a
+# block, several blocks, one dense against the longest and the shortest chunk
+PREV_LENS = (1, 40, 128, 700, 6000, 50000)
+
+
+@pytest.mark.parametrize("d_warp", [0, 1024])
+def test_fast_node2vec_laws_at_chunk_edges(orc, d_warp):
+    g = edge_graph(LENS + PREV_LENS)
+    dg = load(g)
+    if d_warp:
+        dg.set_tuning(d_warp=d_warp)
+    csr = orc.CSR(g)
+    prm = orc.Params(p=4.0, q=3.0, scale=12)
+    pairs = [(i, len(LENS) + j) for i in range(len(LENS)) for j in range(len(PREV_LENS))]
+    # prev itself among cur's entries, so that the return factor is met
+    for i, (cur, pv) in enumerate(pairs):
+        row = g.col[g.row_ptr[cur]:g.row_ptr[cur + 1]]
+        if i % 2:
+            pairs[i] = (cur, int(row[len(row) // 2]) if g.row_ptr[row[len(row) // 2] + 1] > g.row_ptr[row[len(row) // 2]] else pv)
+    n = N // 4
+    cur = torch.tensor([a for a, _ in pairs], dtype=torch.int32, device="cuda").repeat_interleave(n)
+    prev = torch.tensor([b for _, b in pairs], dtype=torch.int32, device="cuda").repeat_interleave(n)
+    paths, plen = dg.walk("node2vec", cur, 2, 20240502 + d_warp, mode="fast", p=4.0, q=3.0, prev=prev,
+                          step0=torch.ones_like(cur))
+    dg.stats()
+    nxt = paths[:, 1].view(len(pairs), n).cpu().numpy()
+    for i, (c, b) in enumerate(pairs):
+        row = g.col[g.row_ptr[c]:g.row_ptr[c + 1]]
+        law = orc.transition(csr, "node2vec", prm, c, b, 1, mode="fast")
+        at = np.searchsorted(row, nxt[i])
+        assert (at < len(row)).all() and (row[at] == nxt[i]).all(), (c, b)
+        _, p = chi2_tv(np.bincount(at, minlength=len(row)), law / law.sum(), n)
+        assert p > P_MIN, (len(row), b, p)
