@@ -58,4 +58,25 @@ cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int6
                       : launch_as<false, false>(g, reqs, n_req, total, cursor, counters, tu, stream));
 }
 
+cudaError_t launch_fast_serve(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tu,
+                              cudaStream_t stream) {
+    auto kern = fast_kernel<true, true, true>;
+    // One 768-thread CTA fills an SM (24 warps of 80 registers), so that the
+    // eight SMs left out below are wholly free for other streams' kernels.
+    // Filling every SM would hold those back for as long as the server runs,
+    // and through the hardware queues streams share, the server's own copies
+    // queued behind them.
+    const int warps = 24;
+    const int sw = max(1, min(SW_MAX, tu.slots / (tu.block_threads / 32)));
+    const size_t smem = cta_smem<true>(warps, sw);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = engine_grid(kern, warps * 32, smem, tu, &sms, &per_sm);
+    if (e != cudaSuccess) return e;
+    ReqTable tab;
+    memset(&tab, 0, sizeof tab);
+    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters};
+    kern<<<(unsigned)(sms - min(8, sms - 1)), warps * 32, smem, stream>>>(g, tab, L, sw, tu.d_warp, sv);
+    return cudaGetLastError();
+}
+
 }  // namespace fw

@@ -169,9 +169,11 @@ inline cudaError_t launch_walk(const GraphDev& g, int mode, const ReqTable& reqs
 cudaError_t launch_serve(const GraphDev& g, int mode, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
                          cudaStream_t stream);
 
-// The fast-mode launch of requests without node2vec (fw_fast.cu).
+// The fast-mode launches (fw_fast.cu).
 cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                         unsigned long long* counters, const Tuning& tune, cudaStream_t stream);
+cudaError_t launch_fast_serve(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
+                              cudaStream_t stream);
 
 Tuning default_tuning();
 Tuning sanitize_tuning(Tuning t);

@@ -1851,16 +1851,11 @@ cudaError_t launch_serve(const GraphDev& g, int mode, const ServeDev& sv, Scratc
                          cudaStream_t stream) {
     const Tuning tu = sanitize_tuning(tune);
     const bool exact = mode == FW_EXACT;
+    if (!exact) return launch_fast_serve(g, sv, scratch, tu, stream);
     switch (tu.block_threads) {
-        case 128:
-            return exact ? launch_serve_one<MODE_EXACT, 128>(g, sv, scratch, tu, stream)
-                         : launch_serve_one<MODE_FAST, 128>(g, sv, scratch, tu, stream);
-        case 512:
-            return exact ? launch_serve_one<MODE_EXACT, 512>(g, sv, scratch, tu, stream)
-                         : launch_serve_one<MODE_FAST, 512>(g, sv, scratch, tu, stream);
-        default:
-            return exact ? launch_serve_one<MODE_EXACT, 256>(g, sv, scratch, tu, stream)
-                         : launch_serve_one<MODE_FAST, 256>(g, sv, scratch, tu, stream);
+        case 128: return launch_serve_one<MODE_EXACT, 128>(g, sv, scratch, tu, stream);
+        case 512: return launch_serve_one<MODE_EXACT, 512>(g, sv, scratch, tu, stream);
+        default: return launch_serve_one<MODE_EXACT, 256>(g, sv, scratch, tu, stream);
     }
 }
 
