@@ -107,12 +107,12 @@ typedef struct {
 /*
  * Engine tuning (Section 5.1's |P_L| and d_t and the launch shape).
  *   block_threads   threads per CTA: 128, 256 or 512 (anything else: the
- *                   default, 512).
+ *                   default, 512, which leaves the shape to the engine while
+ *                   ctas_per_sm is 0 too).
  *   slots           walks resident per CTA: the local task pool P_L, at most
  *                   8 per warp (default 4 per warp).
  *   d_warp          degree threshold d_t: rows with d <= d_warp are sampled
- *                   by one warp, larger rows by the whole CTA (default 65536;
- *                   exact mode caps it at 8184).
+ *                   by one warp, larger rows by the whole CTA (default 65536).
  *   ctas_per_sm     persistent CTAs per SM (0 = as many as fit).
  * Zero fields mean "default".  No field changes a walk's result: exact mode is
  * bit-identical to the CPU oracle under every tuning, and fast mode draws each

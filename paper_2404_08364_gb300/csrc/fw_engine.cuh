@@ -25,6 +25,15 @@
 // merged by an arg-min over race times (a 64-bit atomicMin of packed (time,
 // index) across the warps of a hub task).
 //
+// Exact mode: W = the sum of integer weights, r = floor(x * W / 2^64) from the
+// step's 64-bit Philox draw, pick = smallest i with inclusive prefix > r
+// (inverse transform sampling).  The scan keeps the totals of up to 64 runs of
+// 512-entry pairs in shared memory and only the run holding the crossing is
+// scanned again (a row of one pair is picked from at once).  Measured on the
+// R-MAT-20 node2vec batch of 2^15 walks: 69.8 ms with per-128-entry sums, rows
+// above 8,184 entries as hub tasks and 136 KB of code (the warps waited for
+// instructions 55 % of their time), 12.7 ms on this engine.
+//
 // First-order rules (weighted, MetaPath, PPR) need a row's weights (and
 // labels) and the one picked column, so only those are read: 4 (5) bytes per
 // entry.  A lane takes four 16-byte quads of 512 entries straight into
@@ -42,9 +51,9 @@
 namespace fw {
 namespace {
 
-constexpr int SW_MAX = 8;         // walk slots per warp, upper bound
 constexpr int NHUB = 4;           // hub tasks open at once per CTA
 constexpr int NSEG_MAX = 64;      // segments per hub task
+constexpr int kSums = 64;         // exact mode: run totals per scan
 // A row is cut into segments of kSegQuads quads (16384 entries, counted from
 // its first aligned 16-entry group), or more for rows past NSEG_MAX such
 // segments.  In fast mode segment j draws from random stream j and the step
@@ -116,9 +125,12 @@ struct Area {
     static constexpr int BYTES = HEAD + kWarpHeadBytes;
 };
 
-template <bool N2V>
+// After the warps' areas and the slots, exact mode keeps the run totals of each
+// warp's scan and the segment totals of the hub tasks.
+template <bool EXACT, bool N2V>
 constexpr size_t cta_smem(int warps, int sw) {
-    return (size_t)kHeadBytes + (size_t)warps * ((size_t)sw * sizeof(Slot) + Area<N2V>::BYTES);
+    return (size_t)kHeadBytes + (size_t)warps * ((size_t)sw * sizeof(Slot) + Area<N2V>::BYTES) +
+           (EXACT ? (size_t)(warps * kSums + NHUB * NSEG_MAX) * 8 : 0);
 }
 
 // A warp's weighted reservoir (exponential race with exponential jumps), run
@@ -289,6 +301,105 @@ __device__ __forceinline__ void offer_pair(Res& R, float (&w)[16], bool two, int
         tot = t1;
         own = own1;
     }
+}
+
+// Exact mode: W = the sum of the integer weights, r = floor(x W / 2^64) from
+// the step's 64-bit Philox draw x, the pick = the first entry whose inclusive
+// prefix exceeds r.  A scan keeps the totals of up to kSums runs of `div` pairs
+// in shared memory; the run that r falls into is scanned again, until it is
+// one pair, which is picked from.  A row of one pair is picked from at once.
+struct ExactScan {
+    unsigned long long W;      // sum of the weights scanned
+    unsigned long long x;      // the step's draw
+    unsigned long long r;      // r less the prefix before the range (once known)
+    unsigned long long* sums;  // kSums run totals (shared memory)
+    int div, np;               // pairs per run, pairs scanned
+    bool pick, known;          // pick from the (single) pair; r is known
+    int sel;                   // the picked row index, -1: none
+};
+
+// Sum over the warp of values below 2^36.
+__device__ __forceinline__ unsigned long long warp_total(unsigned long long v) {
+    const unsigned lo = __reduce_add_sync(FULL, (unsigned)v & 0xFFFFFFu);
+    const unsigned hi = __reduce_add_sync(FULL, (unsigned)(v >> 24));
+    return ((unsigned long long)hi << 24) + lo;
+}
+
+// Offer one pair (w: bit patterns of uint32 weights, ordered as load_pair
+// leaves them: quad k of lane l holds entries 128 k + 4 l + j).
+__device__ __forceinline__ void exact_pair(ExactScan& A, const float (&w)[16], int r0, int lane) {
+    unsigned long long q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        q[k] = ((unsigned long long)__float_as_uint(w[4 * k]) + __float_as_uint(w[4 * k + 1])) +
+               ((unsigned long long)__float_as_uint(w[4 * k + 2]) + __float_as_uint(w[4 * k + 3]));
+    const unsigned long long tot = warp_total((q[0] + q[1]) + (q[2] + q[3]));
+    A.W += tot;
+    if (!A.pick) {
+        if (lane == 0) A.sums[A.div == 1 ? A.np : A.np / A.div] += tot;
+        ++A.np;
+        return;
+    }
+    if (!A.known) A.r = __umul64hi(A.x, tot);
+    if (tot == 0) return;
+    // the 128-entry half that holds the crossing, then the lane, then the entry
+    unsigned long long r = A.r;
+    unsigned long long mine = q[3];
+    unsigned e[4] = {__float_as_uint(w[12]), __float_as_uint(w[13]), __float_as_uint(w[14]), __float_as_uint(w[15])};
+    int half = 3;
+    bool found = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const unsigned long long gk = warp_total(q[k]);
+        if (!found) {
+            if (r < gk) {
+                found = true;
+                half = k;
+                mine = q[k];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) e[j] = __float_as_uint(w[4 * k + j]);
+            } else {
+                r -= gk;
+            }
+        }
+    }
+    unsigned long long incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long n = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += n;
+    }
+    const unsigned m = __ballot_sync(FULL, incl > r);
+    const int L = m ? __ffs(m) - 1 : 31;  // (always found, as r < tot)
+    r -= incl - mine;
+    int j = 3;
+    if (r < (unsigned long long)e[0]) j = 0;
+    else if (r < (unsigned long long)e[0] + e[1]) j = 1;
+    else if (r < (unsigned long long)e[0] + e[1] + e[2]) j = 2;
+    A.sel = r0 + half * 128 + 4 * L + __shfl_sync(FULL, j, L);
+}
+
+// Which of the n sums (in shared memory) holds the crossing of r, r less the
+// sums before it; -1 if none.  Warp-collective.
+__device__ __noinline__ int find_crossing(const unsigned long long* sums, int n, unsigned long long& r, int lane) {
+#pragma unroll 1
+    for (int base = 0; base < n; base += 32) {
+        const unsigned long long v = base + lane < n ? sums[base + lane] : 0ull;
+        unsigned long long incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const unsigned m = __ballot_sync(FULL, incl > r);
+        if (m) {
+            const int L = __ffs(m) - 1;
+            r -= __shfl_sync(FULL, incl - v, L);
+            return base + L;
+        }
+        r -= __shfl_sync(FULL, incl, 31);
+    }
+    return -1;
 }
 
 // One lane's quad at row index rel whose last entries lie past the end of the
@@ -533,13 +644,14 @@ __device__ __forceinline__ int chunk_members(const int32_t* __restrict__ B, int 
 
 // Scan the entries of row indices [r_a, lim) of slot sl's row (r_a a multiple
 // of 16 in the CSR arrays, down to -15) as random stream `stream`: weights with
-// the rule's factors, offered to the warp's reservoir R.  False if a copy never
-// landed.  Warp-collective.
-template <bool N2V, bool LAB>
+// the rule's factors, offered to the warp's reservoir R (fast mode) or sums X
+// (exact mode).  False if a copy never landed.  Warp-collective.
+template <bool EXACT, bool N2V, bool LAB>
 __device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, int r_a, int lim, int lane,
-                                           unsigned char* area, uint32_t& ph, Res& R, int stream) {
+                                           unsigned char* area, uint32_t& ph, Res& R, ExactScan& X, int stream) {
     const long long beg = sl.row[0];
-    const float* wrow = g.w_f32 + beg;
+    // (exact mode moves the bit patterns of the integer weights about)
+    const float* wrow = (EXACT ? reinterpret_cast<const float*>(g.w_u32) : g.w_f32) + beg;
     const int algo = sl.rq.algo;
     const int8_t* lrow = nullptr;
     int want = 0;
@@ -614,6 +726,7 @@ __device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, in
             load_pair<LAB>(wrow, lrow, want, rp, lim, left, lane, w);
             if (n2v) {
                 const float f1 = sl.rq.fac_f[1], f2 = sl.rq.fac_f[2];
+                const unsigned i1 = sl.rq.fac_i[1], i2 = sl.rq.fac_i[2];
                 unsigned mk[4] = {0u, 0u, 0u, 0u};
                 if (some) {
                     const unsigned* mw = reinterpret_cast<const unsigned*>(area + Area<N2V>::MASK + (rp - r0)) + lane;
@@ -621,19 +734,25 @@ __device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, in
                     for (int k = 0; k < 4; ++k) mk[k] = mw[32 * k];
                 }
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    w[j] = __fmul_rn(w[j], mk[j >> 2] >> (8 * (j & 3)) & 1u ? f1 : f2);
+                for (int j = 0; j < 16; ++j) {
+                    const bool in = mk[j >> 2] >> (8 * (j & 3)) & 1u;
+                    if (EXACT) w[j] = __uint_as_float(__float_as_uint(w[j]) * (in ? i1 : i2));
+                    else w[j] = __fmul_rn(w[j], in ? f1 : f2);
+                }
                 const int pp = prevpos - (rp - r0);
                 if (prevpos >= 0 && (unsigned)pp < (unsigned)PAIR) {
                     // the return factor in place of the other two
-                    const float wp = __fmul_rn(__ldg(wrow + rp + pp), sl.rq.fac_f[0]);
+                    float wp = __ldg(wrow + rp + pp);
+                    if (EXACT) wp = __uint_as_float(__float_as_uint(wp) * sl.rq.fac_i[0]);
+                    else wp = __fmul_rn(wp, sl.rq.fac_f[0]);
                     const int jp = (pp >> 2 & 31) == lane ? (pp >> 7) * 4 + (pp & 3) : -1;
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         if (j == jp) w[j] = wp;
                 }
             }
-            offer_pair(R, w, rp + STAGE < lim, rp, lane, sl, stream);
+            if (EXACT) exact_pair(X, w, rp, lane);
+            else offer_pair(R, w, rp + STAGE < lim, rp, lane, sl, stream);
         }
         if (N2V) __syncwarp();  // the membership bytes are cleared for the next chunk
     }
@@ -736,6 +855,12 @@ __device__ __noinline__ int hub_claim(CtaHead& H0, int lane) {
         __threadfence_block();
     }
     return __shfl_sync(FULL, got, 0);
+}
+
+// The step's 64-bit draw (exact mode).
+__device__ __noinline__ unsigned long long step_draw(const Slot& s) {
+    const uint4 o = step_block(s.rq.seed, (uint64_t)(s.rq.q_id0 + s.q), (uint32_t)s.t);
+    return (unsigned long long)o.x | (unsigned long long)o.y << 32;
 }
 
 // What the engine's out-of-line parts share.
@@ -957,12 +1082,12 @@ __device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restric
 // them is smaller: see the instruction cache above).
 // SERVE: the served form's build (queries claimed from the request ring,
 // completion stamps, idle polling); the batch build compiles all of that out.
-template <bool N2V, bool LAB, bool SERVE>
+template <bool EXACT, bool N2V, bool LAB, bool SERVE>
 // Registers: 64 a thread for first-order launches (32 warps per SM), 80 for
 // node2vec (24 warps; 128 registers and 16 warps measured 241 ms against 202
 // on the R-MAT-25 batch of 2^18 walks, 64 registers with spills 248).
 __global__ void __maxnreg__(N2V ? 80 : 64)
-    fast_kernel(const __grid_constant__ GraphDev g, const __grid_constant__ ReqTable tab, const __grid_constant__ Launch L,
+    walk_kernel(const __grid_constant__ GraphDev g, const __grid_constant__ ReqTable tab, const __grid_constant__ Launch L,
                 int sw, int d_t, const __grid_constant__ ServeDev sv) {
     const ReqDev* __restrict__ reqs = SERVE ? sv.ring : (L.reqs ? L.reqs : tab.r);
     extern __shared__ __align__(128) unsigned char dyn[];
@@ -970,6 +1095,7 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
     CtaHead& head = *reinterpret_cast<CtaHead*>(dyn);
     unsigned char* area = dyn + kHeadBytes + warp * Area<N2V>::BYTES;
     Slot* slots = reinterpret_cast<Slot*>(dyn + kHeadBytes + nwarp * Area<N2V>::BYTES);
+    unsigned long long* hub_sums = reinterpret_cast<unsigned long long*>(slots + nwarp * sw);
     WarpHead& wh = *reinterpret_cast<WarpHead*>(area + Area<N2V>::HEAD);
     uint32_t ph = 0;  // parity at which the next chunk's columns land
     if (N2V && lane == 0) {
@@ -1033,32 +1159,28 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
         }
 
         // ------------------------------------ stream the row range (one site)
-        // A hub segment is one range.  A row sampled by this warp alone is
-        // cut into the hub path's segments, segment j drawing from random
-        // stream j, and the step keeps the smallest (race time, index) over
-        // them, as a hub task's merge does.
-        unsigned long long best = ~0ull;
+        int sel = -1;        // the picked row index
+        bool fin = true;     // the step is done
         bool scanned = true;
+        if (!EXACT) {
+            // A hub segment is one range.  A row sampled by this warp alone is
+            // cut into the hub path's segments, segment j drawing from random
+            // stream j, and the step keeps the smallest (race time, index)
+            // over them, as a hub task's merge does.
+            unsigned long long best = ~0ull;
+            ExactScan none;
 #pragma unroll 1
-        for (; ra < lim; ra += sq) {
-            Res R;
-            R.init();
-            if (!scan_range<N2V, LAB>(g, sl, ra, min(lim, ra + sq), lane, area, ph, R, stream)) {
-                scanned = false;
-                break;
+            for (; ra < lim; ra += sq) {
+                Res R;
+                R.init();
+                if (!scan_range<EXACT, N2V, LAB>(g, sl, ra, min(lim, ra + sq), lane, area, ph, R, none, stream)) {
+                    scanned = false;
+                    break;
+                }
+                if (R.sel >= 0) best = min(best, race_key(R));
+                ++stream;
             }
-            if (R.sel >= 0) best = min(best, race_key(R));
-            ++stream;
-        }
-        if (N2V && !scanned) {
-            if (lane == 0) atomicAdd(&L.counters[C_TIMEOUT], 1ull);
-            break;
-        }
-
-        // ------------------------------------------------ use the result
-        if (lane == 0) {
-            bool fin = true;
-            if (seg >= 0) {
+            if (seg >= 0 && lane == 0) {
                 // fold the segment into its hub task; the warp that completes
                 // the last segment finishes the step
                 HubTask& H = head.hub[seg >> 8];
@@ -1068,18 +1190,91 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
                 __threadfence_block();
                 best = *(volatile unsigned long long*)&H.best;
             }
-            if (fin) {
-                if (best == ~0ull) {
-                    __threadfence_block();
-                    *(volatile int*)&sl.state = ST_FINISH;  // nothing selectable: the walk stops here
-                } else {
-                    count_step(wh.cnt, (int)(sl.row[1] - sl.row[0]), sl.rq.algo, seg >= 0);
-                    commit(g, sl, (int)(best & 0xFFFFFFFFull), seg >= 0);
+            sel = best == ~0ull ? -1 : (int)(best & 0xFFFFFFFFull);
+        } else if (ra < lim) {
+            // Sums first, then the run of pairs that r falls into, down to one
+            // pair.  A hub segment only adds its total to the task; the warp
+            // that completes the last one goes on in the segment of the pick.
+            ExactScan X;
+            X.sums = hub_sums + NHUB * NSEG_MAX + warp * kSums;
+            X.known = false;
+            X.sel = -1;
+            bool sums_only = seg >= 0;
+            if (!sums_only) X.x = step_draw(sl);
+#pragma unroll 1
+            for (;;) {
+                const int np = (lim - ra + PAIR - 1) / PAIR;
+                X.pick = np == 1 && !sums_only;
+                X.div = (np + kSums - 1) / kSums;
+                X.np = 0;
+                X.W = 0;
+                X.sums[lane] = 0;
+                X.sums[32 + lane] = 0;
+                __syncwarp();
+                Res none;
+                if (!scan_range<EXACT, N2V, LAB>(g, sl, ra, lim, lane, area, ph, none, X, 0)) {
+                    scanned = false;
+                    break;
                 }
-                if (seg >= 0) {
-                    __threadfence_block();
-                    atomicExch(&head.hub[seg >> 8].ctl, H_FREE);
+                __syncwarp();
+                if (X.pick) break;
+                if (sums_only) {
+                    sums_only = false;
+                    HubTask& H = head.hub[seg >> 8];
+                    unsigned long long* hs = hub_sums + (seg >> 8) * NSEG_MAX;
+                    const int nseg = hub_nseg(*(volatile unsigned*)&H.ctl);
+                    int last = 0;
+                    if (lane == 0) {
+                        hs[stream] = X.W;
+                        __threadfence_block();
+                        last = atomicAdd(&H.done_seg, 1) == nseg - 1;
+                        __threadfence_block();
+                    }
+                    if (!__shfl_sync(FULL, last, 0)) {
+                        fin = false;
+                        break;
+                    }
+                    unsigned long long W = 0;
+                    for (int i = 0; i < nseg; ++i) W += *(volatile unsigned long long*)&hs[i];
+                    if (W == 0) break;
+                    X.r = __umul64hi(step_draw(sl), W);
+                    X.known = true;
+                    const int i = find_crossing(hs, nseg, X.r, lane);
+                    if (i < 0) break;  // never, as r < W
+                    ra = -(int)(sl.row[0] & 15) + i * sq;
+                    lim = min((int)(sl.row[1] - sl.row[0]), ra + sq);
+                    continue;
                 }
+                if (!X.known) {
+                    if (X.W == 0) break;
+                    X.r = __umul64hi(X.x, X.W);
+                    X.known = true;
+                }
+                const int i = find_crossing(X.sums, kSums, X.r, lane);
+                if (i < 0) break;  // never, as r < W
+                ra += i * X.div * PAIR;
+                lim = min(lim, ra + X.div * PAIR);
+                __syncwarp();
+            }
+            sel = X.sel;
+        }
+        if ((EXACT || N2V) && !scanned) {
+            if (lane == 0) atomicAdd(&L.counters[C_TIMEOUT], 1ull);
+            break;
+        }
+
+        // ------------------------------------------------ use the result
+        if (lane == 0 && fin) {
+            if (sel < 0) {
+                __threadfence_block();
+                *(volatile int*)&sl.state = ST_FINISH;  // nothing selectable (or a dead end): the walk stops here
+            } else {
+                count_step(wh.cnt, (int)(sl.row[1] - sl.row[0]), sl.rq.algo, seg >= 0);
+                commit(g, sl, sel, seg >= 0);
+            }
+            if (seg >= 0) {
+                __threadfence_block();
+                atomicExch(&head.hub[seg >> 8].ctl, H_FREE);
             }
         }
         __syncwarp();

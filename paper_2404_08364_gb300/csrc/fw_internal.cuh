@@ -169,11 +169,17 @@ inline cudaError_t launch_walk(const GraphDev& g, int mode, const ReqTable& reqs
 cudaError_t launch_serve(const GraphDev& g, int mode, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
                          cudaStream_t stream);
 
-// The fast-mode launches (fw_fast.cu).
+// The two modes' launches (fw_fast.cu, fw_exact.cu).
 cudaError_t launch_fast(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                         unsigned long long* counters, const Tuning& tune, cudaStream_t stream);
 cudaError_t launch_fast_serve(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
                               cudaStream_t stream);
+cudaError_t launch_exact(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                         unsigned long long* counters, const Tuning& tune, cudaStream_t stream);
+cudaError_t launch_exact_serve(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tune,
+                               cudaStream_t stream);
+
+constexpr int kSlotsPerWarp = 8;  // walk slots per warp, upper bound
 
 Tuning default_tuning();
 Tuning sanitize_tuning(Tuning t);

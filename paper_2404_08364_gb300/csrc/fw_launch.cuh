@@ -1,0 +1,85 @@
+// Launches of the walk engine, instantiated for fast mode in fw_fast.cu and for
+// exact mode in fw_exact.cu (two translation units build in parallel).
+#pragma once
+
+#include <string.h>
+
+#include "fw_engine.cuh"
+
+namespace fw {
+namespace {
+
+// Grid and shared memory of one engine launch: every SM filled as far as the
+// kernel's registers and shared memory allow (at most tu.ctas_per_sm CTAs each).
+template <typename K>
+cudaError_t engine_grid(K kern, int threads, size_t smem, const Tuning& tu, int* sms, int* per_sm) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (*per_sm < 1) return cudaErrorInvalidConfiguration;
+    if (tu.ctas_per_sm > 0) *per_sm = min(*per_sm, tu.ctas_per_sm);
+    return cudaSuccess;
+}
+
+template <bool EXACT, bool N2V, bool LAB>
+cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                      unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
+    auto kern = walk_kernel<EXACT, N2V, LAB, false>;
+    const int sw = max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
+    // CTAs of 256 threads unless the caller chose: at 80 registers three of
+    // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
+    // (R-MAT-25 node2vec: 240 -> 202 ms), and a hub row's last segments hold
+    // back 8 warps instead of 16 (PPR from the R-MAT-22 hub: 5.7 -> 4.8 ms).
+    const int threads = tu.own_shape || tu.ctas_per_sm > 0 ? tu.block_threads : 256;
+    const int warps = threads / 32;
+    const size_t smem = cta_smem<EXACT, N2V>(warps, sw);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = engine_grid(kern, threads, smem, tu, &sms, &per_sm);
+    if (e != cudaSuccess) return e;
+    const int64_t per_cta = (int64_t)sw * warps;
+    const int64_t grid = min((int64_t)sms * per_sm, (total + per_cta - 1) / per_cta);
+    ServeDev none;
+    memset(&none, 0, sizeof none);
+    // (a table inside the parameter block is found by the kernel itself)
+    const Launch L = {reqs.ext, n_req, (long long)total, cursor, counters};
+    kern<<<(unsigned)grid, threads, smem, stream>>>(g, reqs, L, sw, tu.d_warp, none);
+    return cudaGetLastError();
+}
+
+template <bool EXACT>
+cudaError_t launch_mode(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
+                        unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
+    const bool n2v = reqs.algos >> FW_NODE2VEC & 1u, lab = reqs.algos >> FW_METAPATH & 1u;
+    return n2v ? (lab ? launch_as<EXACT, true, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
+                      : launch_as<EXACT, true, false>(g, reqs, n_req, total, cursor, counters, tu, stream))
+               : (lab ? launch_as<EXACT, false, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
+                      : launch_as<EXACT, false, false>(g, reqs, n_req, total, cursor, counters, tu, stream));
+}
+
+template <bool EXACT>
+cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tu, cudaStream_t stream) {
+    auto kern = walk_kernel<EXACT, true, true, true>;
+    // One 768-thread CTA fills an SM (24 warps of 80 registers), so that the
+    // eight SMs left out below are wholly free for other streams' kernels.
+    // Filling every SM would hold those back for as long as the server runs,
+    // and through the hardware queues streams share, the server's own copies
+    // queued behind them.
+    const int warps = 24;
+    const int sw = max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
+    const size_t smem = cta_smem<EXACT, true>(warps, sw);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = engine_grid(kern, warps * 32, smem, tu, &sms, &per_sm);
+    if (e != cudaSuccess) return e;
+    ReqTable tab;
+    memset(&tab, 0, sizeof tab);
+    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters};
+    kern<<<(unsigned)(sms - min(8, sms - 1)), warps * 32, smem, stream>>>(g, tab, L, sw, tu.d_warp, sv);
+    return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace fw

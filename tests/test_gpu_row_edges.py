@@ -106,3 +106,29 @@ def test_fast_node2vec_laws_at_chunk_edges(orc, d_warp):
         assert (at < len(row)).all() and (row[at] == nxt[i]).all(), (c, b)
         _, p = chi2_tv(np.bincount(at, minlength=len(row)), law / law.sum(), n)
         assert p > P_MIN, (len(row), b, p)
+
+
+@pytest.mark.parametrize("algo", ["weighted", "node2vec", "metapath", "ppr"])
+@pytest.mark.parametrize("d_warp", [0, 1024])
+def test_exact_picks_at_tile_edges(orc, algo, d_warp):
+    """Exact mode on the same rows (and one of 40,000 entries, which is summed
+    in runs of two pairs): bit-equal to the oracle."""
+    g = edge_graph(LENS + PREV_LENS + (40000,))
+    dg = load(g)
+    if d_warp:
+        dg.set_tuning(d_warp=d_warp)
+    rows = len(LENS) + len(PREV_LENS) + 1
+    starts = torch.arange(rows, dtype=torch.int32).repeat_interleave(96)
+    kw = {}
+    if algo == "node2vec":
+        # prev goes over all rows too, and every third walk over cur's own middle entry
+        mid = torch.from_numpy(g.col)[torch.from_numpy(g.row_ptr[:rows] + np.diff(g.row_ptr[:rows + 1]) // 2)]
+        i = torch.arange(starts.numel())
+        kw["prev"] = torch.where(i % 3 == 0, mid[starts.long()], ((i * 7) % rows).to(torch.int32))
+    prm = orc.Params(p=2.0, q=0.5, schema=(2, 4), ppr_stop=0.5)
+    rp, rl = orc.walk_exact(orc.CSR(g), algo, prm, starts.numpy(), 2, 77, **{k: v.numpy() for k, v in kw.items()})
+    paths, plen = dg.walk(algo, starts.cuda(), 2, 77, mode="exact", p=2.0, q=0.5, schema=(2, 4), ppr_stop=0.5,
+                          **{k: v.cuda() for k, v in kw.items()})
+    dg.stats()
+    assert np.array_equal(plen.cpu().numpy(), rl)
+    assert np.array_equal(paths.cpu().numpy(), rp)
