@@ -57,7 +57,6 @@ struct fw_graph {
     int device;
     GraphDev g;
     bool owned;
-    int64_t d_max;
     uint32_t max_w_u32;
     Scratch* scratch;          // device: cursor + counters
     Tuning tuning;
@@ -256,7 +255,7 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
         release(G);
         return fail(FW_ECUDA, "fw_load_csr: checks: %s", cudaGetErrorString(e));
     }
-    G->d_max = (int64_t)co.d_max;
+    G->g.d_max = (int64_t)co.d_max;
     G->max_w_u32 = co.max_w_u32;
     // offsets and column ranges are always enforced: the kernels index by them
     if (ends[0] != 0 || ends[1] != m || (co.flags & V_ROWPTR)) rc = fail(FW_EINVAL, "fw_load_csr: row_ptr not monotone from 0 to m");
@@ -281,7 +280,7 @@ extern "C" int fw_graph_info(const fw_graph* g, int64_t* n, int64_t* m, int64_t*
     if (!g) return fail(FW_EINVAL, "fw_graph_info: NULL graph");
     if (n) *n = g->g.n;
     if (m) *m = g->g.m;
-    if (d_max) *d_max = g->d_max;
+    if (d_max) *d_max = g->g.d_max;
     if (has_f32) *has_f32 = g->g.w_f32 != nullptr;
     if (has_u32) *has_u32 = g->g.w_u32 != nullptr;
     if (has_type) *has_type = g->g.etype != nullptr;
@@ -291,7 +290,7 @@ extern "C" int fw_graph_info(const fw_graph* g, int64_t* n, int64_t* m, int64_t*
 extern "C" int fw_set_tuning(fw_graph* g, const fw_tuning* t) {
     if (!g) return fail(FW_EINVAL, "fw_set_tuning: NULL graph");
     Tuning tu = default_tuning();
-    if (t) tu = Tuning{t->block_threads, t->slots, t->d_warp, t->ctas_per_sm, true};
+    if (t) tu = Tuning{t->block_threads, t->slots, t->d_warp, t->ctas_per_sm, true, true};
     g->tuning = sanitize_tuning(tu);
     return FW_OK;
 }

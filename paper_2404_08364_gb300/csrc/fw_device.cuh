@@ -72,6 +72,11 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
         : "memory");
 }
 
+// Start fetching `bytes` (a multiple of 16) from a 16-byte boundary into L2.
+__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Orders this thread's ordinary shared-memory stores before later bulk copies
 // into the same bytes.
 __device__ __forceinline__ void fence_proxy_async_cta() {

@@ -99,6 +99,7 @@ struct __align__(16) Slot {
 struct CtaHead {
     HubTask hub[NHUB];
     int hub_open;       // hub tasks with segments left to hand out (a hint: claims decide)
+    int working;        // warps that may still hold walks
     int abort_flag;
 };
 
@@ -108,6 +109,7 @@ struct WarpHead {
     unsigned long long idle_since;  // when the warp ran out of work (0: it has some)
     unsigned nap;                   // idle back-off (ns)
     int exhausted;                  // no query is left to claim
+    int done;                       // no walk is left either (not counted in CtaHead::working)
 };
 constexpr int kHeadBytes = (sizeof(CtaHead) + 127) & ~127;
 constexpr int kWarpHeadBytes = (sizeof(WarpHead) + 127) & ~127;
@@ -172,11 +174,12 @@ __device__ __forceinline__ unsigned long long race_key(const Res& r) {
 }
 
 // Entries per segment of a row of d entries whose first aligned 16-entry group
-// starts at row index r_a: kSegQuads quads, or more for rows of more than
-// NSEG_MAX such segments; a multiple of 32 quads (one quad per lane).
-__device__ __forceinline__ int seg_entries(int r_a, int d) {
+// starts at row index r_a: seg_q quads (kSegQuads in fast mode, whose random
+// streams are the segments'), or more for rows of more than NSEG_MAX such
+// segments; a multiple of 32 quads (one quad per lane).
+__device__ __forceinline__ int seg_entries(int r_a, int d, int seg_q) {
     const unsigned nq = ((unsigned)(d - r_a) + 3) >> 2;
-    const unsigned sq = max((unsigned)kSegQuads, (nq + NSEG_MAX - 1) / NSEG_MAX);
+    const unsigned sq = max((unsigned)seg_q, (nq + NSEG_MAX - 1) / NSEG_MAX);
     return (int)(((sq + 31) & ~31u) << 2);
 }
 
@@ -718,6 +721,9 @@ __device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, in
                 const int rn = r0 + CHUNK, k = min(min(CHUNK, (lim - rn + 15) & ~15), whole - rn);
                 mbar_arrive_expect_tx(bar, (uint32_t)max(k, 0) * 4u);
                 if (k > 0) tma_load_1d(col, g.col + beg + rn, (uint32_t)k * 4u, bar);
+                // a long row's weights are asked for a chunk ahead too (R-MAT-25
+                // batch: 197.6 -> 190.1 ms)
+                if (k == CHUNK) prefetch_l2(wrow + rn, CHUNK * 4);
             }
         }
 #pragma unroll 1
@@ -870,6 +876,9 @@ struct Launch {
     long long total;
     unsigned long long* cursor;
     unsigned long long* counters;
+    int claimers;   // warps of a CTA that claim queries (the others only help with hub tasks)
+    int seg_q;      // exact mode: quads per hub segment
+    unsigned nap;   // sleep of a warp that has no walk left between looks for hub work (ns); 0: it returns
 };
 
 // Claim one query for the empty slot sl: the slot's new state, ST_EMPTY if
@@ -1048,23 +1057,45 @@ __device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restric
         if (st == ST_HUB) waiting = true;
         if (st == ST_READY) return jj;
     }
-    // Nothing to do now.  Batch: done once every slot is empty.  Served: poll
-    // for new requests; return once the host asks to stop.  Either way a wait
-    // lasts 2 s at most.
-    if (!waiting && !SERVE) return PICK_QUIT;
+    // Nothing to do now.  Either way a wait lasts 2 s at most.
+    if (!SERVE && !waiting) {
+        // Batch: no walk is left to claim.  The warp stays to help with hub
+        // tasks until no warp of the CTA holds a walk, in a loop of its own
+        // that takes few issue slots from the warps that are scanning.
+        if (!L.nap) return PICK_QUIT;
+        int quit = 0;
+        if (lane == 0) {
+            if (!wh.done) {
+                wh.done = 1;
+                atomicSub(&head.working, 1);
+            }
+            const unsigned long long t0 = global_timer_ns();
+#pragma unroll 1
+            while (*(volatile int*)&head.hub_open <= 0) {
+                quit = *(volatile int*)&head.working <= 0 || *(volatile int*)&head.abort_flag ||
+                       global_timer_ns() - t0 > kWaitLimitNs;
+                if (quit) break;
+                __nanosleep(L.nap);
+            }
+        }
+        return __shfl_sync(FULL, quit, 0) ? PICK_QUIT : PICK_AGAIN;
+    }
+    // Walks parked at hub tasks: help (the caller looks for hub work first) or
+    // wait for them.  Served: poll for new requests; return once the host asks
+    // to stop.
     int quit = 0;
     if (lane == 0) {
         const unsigned long long now = global_timer_ns();
         if (wh.idle_since == 0) wh.idle_since = now;
         const bool late = now - wh.idle_since > kWaitLimitNs;
-        if (!waiting) {
-            quit = late || *sv.stop;
-        } else {
+        if (waiting) {
             if (late) {
                 atomicAdd(&L.counters[C_TIMEOUT], 1ull);
                 head.abort_flag = 1;
             }
             quit = *(volatile int*)&head.abort_flag;
+        } else {
+            quit = late || *sv.stop;
         }
     }
     if (__shfl_sync(FULL, quit, 0)) return PICK_QUIT;
@@ -1108,11 +1139,13 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
     if (lane == 0) {
         wh.idle_since = 0;
         wh.nap = 128;
-        wh.exhausted = 0;
+        wh.exhausted = warp >= L.claimers;
+        wh.done = warp >= L.claimers;
     }
     if (threadIdx.x < NHUB) head.hub[threadIdx.x].ctl = H_FREE;
     if (threadIdx.x == 0) {
         head.hub_open = 0;
+        head.working = min(L.claimers, nwarp);
         head.abort_flag = 0;
     }
     __syncthreads();
@@ -1143,7 +1176,7 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
         int lim = (int)(sl.row[1] - sl.row[0]);
         int ra = lim ? -(int)(sl.row[0] & 15) : 0;  // the scan starts on a 16-entry group (a dead end has none)
         int stream = 0;
-        const int sq = seg_entries(ra, lim);
+        const int sq = seg_entries(ra, lim, EXACT ? L.seg_q : kSegQuads);
         if (seg >= 0) {
             stream = seg & 0xFF;
             ra += stream * sq;

@@ -84,6 +84,7 @@ struct GraphDev {
     const int8_t* etype;
     int64_t n;
     int64_t m;
+    int64_t d_max;  // longest row
 };
 
 // Counter slots in the device scratch (all uint64).
@@ -148,6 +149,7 @@ struct Tuning {
     int slots;
     int d_warp;
     int ctas_per_sm;
+    bool own_d;      // d_warp was set by the caller
     bool own_shape;  // block_threads was set by the caller (else each engine may take the CTA size that suits it)
 };
 

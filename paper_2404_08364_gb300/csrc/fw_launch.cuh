@@ -34,19 +34,46 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
     // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
     // (R-MAT-25 node2vec: 240 -> 202 ms), and a hub row's last segments hold
     // back 8 warps instead of 16 (PPR from the R-MAT-22 hub: 5.7 -> 4.8 ms).
-    const int threads = tu.own_shape || tu.ctas_per_sm > 0 ? tu.block_threads : 256;
-    const int warps = threads / 32;
-    const size_t smem = cta_smem<EXACT, N2V>(warps, sw);
+    const bool own = tu.own_shape || tu.ctas_per_sm > 0;
+    int threads = own ? tu.block_threads : 256, use = sw;
     int sms = 0, per_sm = 0;
-    cudaError_t e = engine_grid(kern, threads, smem, tu, &sms, &per_sm);
+    cudaError_t e = engine_grid(kern, threads, cta_smem<EXACT, N2V>(threads / 32, sw), tu, &sms, &per_sm);
     if (e != cudaSuccess) return e;
-    const int64_t per_cta = (int64_t)sw * warps;
-    const int64_t grid = min((int64_t)sms * per_sm, (total + per_cta - 1) / per_cta);
+    const int64_t resident = (int64_t)sms * per_sm * (threads / 32);
+    int64_t grid = (int64_t)sms * per_sm;
+    Launch L = {reqs.ext, n_req, (long long)total, cursor, counters, threads / 32, kSegQuads, 4096u};
+    int d_t = tu.d_warp;
+    if (total < resident) {
+        // Fewer walks than resident warps: latency counts.  One walk per warp
+        // (a warp advances its walks one after another), spread evenly over
+        // the CTAs.  Hub rows begin at one segment (fast mode) or where the
+        // pieces are still worth a hand-off (exact mode); where the graph has
+        // such rows, one large CTA per SM keeps warps at hand for them.
+        // Measured (us): 1,000 exact walks of 80 on a 1,000-vertex graph 617
+        // (four walks per warp) -> 222; 32 node2vec walks of 40 on R-MAT-22,
+        // fast 868 -> 777, exact 1,095 -> 712 (helpers); 129 PPR walks on
+        // R-MAT-22 222 -> 201.
+        use = 1;
+        if (!tu.own_d) {
+            d_t = min(d_t, EXACT ? 4096 : 4 * kSegQuads);
+            if (EXACT) L.seg_q = 512;
+        }
+        if (!own && g.d_max > d_t) {
+            threads = 768;
+            e = engine_grid(kern, threads, cta_smem<EXACT, N2V>(threads / 32, use), tu, &sms, &per_sm);
+            if (e != cudaSuccess) return e;
+        }
+        grid = min((int64_t)sms * per_sm, total);
+        L.claimers = (int)((total + grid - 1) / grid);
+        L.nap = 512u;
+    } else {
+        use = (int)min((int64_t)sw, total / resident);
+    }
+    if (g.d_max <= d_t) L.nap = 0u;  // no hub tasks: warps without walks return at once
+    const size_t smem = cta_smem<EXACT, N2V>(threads / 32, use);
     ServeDev none;
     memset(&none, 0, sizeof none);
-    // (a table inside the parameter block is found by the kernel itself)
-    const Launch L = {reqs.ext, n_req, (long long)total, cursor, counters};
-    kern<<<(unsigned)grid, threads, smem, stream>>>(g, reqs, L, sw, tu.d_warp, none);
+    kern<<<(unsigned)grid, threads, smem, stream>>>(g, reqs, L, use, d_t, none);
     return cudaGetLastError();
 }
 
@@ -76,7 +103,7 @@ cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, 
     if (e != cudaSuccess) return e;
     ReqTable tab;
     memset(&tab, 0, sizeof tab);
-    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters};
+    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters, warps, kSegQuads, 0u};
     kern<<<(unsigned)(sms - min(8, sms - 1)), warps * 32, smem, stream>>>(g, tab, L, sw, tu.d_warp, sv);
     return cudaGetLastError();
 }

@@ -3,7 +3,7 @@
 
 namespace fw {
 
-Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false}; }
+Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false, false}; }
 
 Tuning sanitize_tuning(Tuning t) {
     const Tuning d = default_tuning();
@@ -13,7 +13,10 @@ Tuning sanitize_tuning(Tuning t) {
     }
     if (t.slots <= 0) t.slots = 4 * (t.block_threads / 32);  // four walks per warp
     if (t.slots > (t.block_threads / 32) * kSlotsPerWarp) t.slots = (t.block_threads / 32) * kSlotsPerWarp;
-    if (t.d_warp <= 0) t.d_warp = d.d_warp;
+    if (t.d_warp <= 0) {
+        t.d_warp = d.d_warp;
+        t.own_d = false;
+    }
     if (t.d_warp < 128) t.d_warp = 128;
     if (t.d_warp > (1 << 30)) t.d_warp = 1 << 30;
     if (t.ctas_per_sm < 0) t.ctas_per_sm = 0;

@@ -132,3 +132,23 @@ def test_exact_picks_at_tile_edges(orc, algo, d_warp):
     dg.stats()
     assert np.array_equal(plen.cpu().numpy(), rl)
     assert np.array_equal(paths.cpu().numpy(), rp)
+
+
+@pytest.mark.parametrize("mode", ["fast", "exact"])
+@pytest.mark.parametrize("algo", ["weighted", "node2vec", "metapath", "ppr"])
+def test_few_walks_equal_the_same_walks_in_a_large_batch(mode, algo):
+    """Launches of 1, 37 and 200 walks (one walk per warp, helper warps, hub
+    rows from one segment on) against the same queries of a full batch."""
+    import fw_inputs as fi
+    from gpu_common import cached_graph, device_graph
+    g = cached_graph("rmat", 18, 2)
+    dg = device_graph(g)
+    assert dg.info()["d_max"] > 16384
+    starts = fi.random_starts(g.n, 20000, 5, "cuda")
+    starts[:5] = int((g.row_ptr[1:] - g.row_ptr[:-1]).argmax())
+    kw = dict(max_len=12, seed=9, mode=mode, p=2.0, q=0.5)
+    paths, plen = dg.walk(algo, starts, **kw)
+    for q0, n in ((0, 1), (0, 37), (3, 200)):
+        p, l = dg.walk(algo, starts[q0:q0 + n].clone(), q_id0=q0, **kw)
+        dg.stats()
+        assert torch.equal(l, plen[q0:q0 + n]) and torch.equal(p, paths[q0:q0 + n]), (q0, n)
