@@ -40,196 +40,391 @@ __device__ __forceinline__ float unit_open23(uint32_t x) { return ((float)(x >> 
 __device__ __forceinline__ uint4 elem_block(uint64_t seed, uint64_t r, uint32_t j, uint32_t c) {
     return philox4x32_10(make_uint4((uint32_t)r, (uint32_t)(r >> 32), j, c), make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
 }
+
+// The selection test of Alg. 3 and 4, u < w / S, for four elements: bit q of
+// the result.  Rarely by a division: a product u S above w by more than the
+// rounding of either side already says no (the summand keeps denormal weights
+// on the exact test).
+__device__ __forceinline__ unsigned picks(const uint4& x, const float (&w)[4], const float (&S)[4]) {
+    const float u[4] = {unit24(x.x), unit24(x.y), unit24(x.z), unit24(x.w)};
+    bool maybe[4], any = false;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        maybe[q] = w[q] > 0.0f && !(u[q] * S[q] > __fmaf_rn(w[q], 1.000001f, 1e-30f));
+        any = any || maybe[q];
+    }
+    unsigned m = 0;
+    if (any) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (maybe[q] && u[q] < w[q] / S[q]) m |= 1u << q;
+    }
+    return m;
+}
+
 __device__ __forceinline__ uint32_t pick_word(const uint4& b, int i) {
     return (i & 3) == 0 ? b.x : (i & 3) == 1 ? b.y : (i & 3) == 2 ? b.z : b.w;
 }
 
-// Group collectives for K = 32 (shuffles) or K = 256 (shuffles + shared).
+// Four weights of thread j: w[b + q K + j], 0 past n.
+template <int K>
+__device__ __forceinline__ void load4(const float* __restrict__ w, uint32_t n, uint32_t b, uint32_t j, float (&v)[4]) {
+    if (b + 4 * K <= n) {
+        const float* p = w + b + j;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = __ldg(p + q * K);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t e = b + q * K + j;
+            v[q] = 0.0f;
+            if (b + q * K < n && e < n) v[q] = __ldg(w + e);
+        }
+    }
+}
+
+__device__ __forceinline__ float warp_incl_scan(float v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float n = __shfl_up_sync(FULL, v, o);
+        if (lane >= o) v += n;
+    }
+    return v;
+}
+
+// A group of K threads: a warp (K = 32) or a CTA (K = 256, with shared buffers).
 template <int K>
 struct Group {
-    float* fbuf;   // K / 32 floats
-    int* ibuf;     // K / 32 ints
+    float* fbuf;   // 2 x 4 x 8 floats
+    int* ibuf;     // 8 ints
     int tid;
 
-    __device__ __forceinline__ void sync() {
-        if (K == 32) __syncwarp();
-        else __syncthreads();
-    }
-    __device__ __forceinline__ float incl_scan(float v) {
-        const int lane = tid & 31;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float n = __shfl_up_sync(FULL, v, o);
-            if (lane >= o) v += n;
-        }
-        if (K == 32) return v;
-        const int wp = tid >> 5;
-        if (lane == 31) fbuf[wp] = v;
-        __syncthreads();
-        float before = 0.0f;
-        for (int i = 0; i < wp; ++i) before += fbuf[i];
-        __syncthreads();
-        return v + before;
-    }
-    __device__ __forceinline__ float total(float incl) {
-        if (K == 32) return __shfl_sync(FULL, incl, 31);
-        __shared__ float t;
-        if (tid == K - 1) t = incl;
-        __syncthreads();
-        const float r = t;
-        __syncthreads();
-        return r;
-    }
     __device__ __forceinline__ int max_int(int v) {
         v = __reduce_max_sync(FULL, v);
         if (K == 32) return v;
+        __syncthreads();
         if ((tid & 31) == 0) ibuf[tid >> 5] = v;
         __syncthreads();
         int m = ibuf[0];
         for (int i = 1; i < K / 32; ++i) m = max(m, ibuf[i]);
-        __syncthreads();
         return m;
     }
 };
 
+// Inclusive prefix sum of one value per thread over the group.
+template <int K>
+__device__ __forceinline__ float group_scan(Group<K>& G, float v) {
+    const int lane = G.tid & 31, wp = G.tid >> 5;
+    v = warp_incl_scan(v, lane);
+    if (K == 32) return v;
+    __syncthreads();
+    if (lane == 31) G.fbuf[wp] = v;
+    __syncthreads();
+    float before = 0.0f;
+    for (int i = 0; i < wp; ++i) before += G.fbuf[i];
+    return v + before;
+}
+
+// At most one element per thread (n <= K): the selected index is the thread's
+// own, so both algorithms end in one maximum; they differ in how they round
+// the running total.  (On 2^18 draws of 32 weights at warp width the
+// four-element code takes 112 us.)
+template <int K, bool ZIG>
+__device__ int draw_short(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
+    const int j = G.tid;
+    const float v = j < n ? __ldg(w + j) : 0.0f;
+    const float u = unit24(elem_block(seed, r, (uint32_t)j, 0).x);
+    const float incl = group_scan<K>(G, v);
+    const float S = ZIG ? (incl - v) + v : incl;
+    return G.max_int(v > 0.0f && u < v / S ? j : -1);
+}
+
+// ZPRS's result: the selection of the highest thread that selected anything.
+template <int K>
+__device__ __forceinline__ int zprs_winner(Group<K>& G, int C) {
+    const int top = G.max_int(C >= 0 ? G.tid : -1);
+    // broadcast the winner's C (K <= 256: through the group's int buffer)
+    if (K == 32) return top < 0 ? -1 : __shfl_sync(FULL, C, top);
+    __syncthreads();
+    if (G.tid == top) G.ibuf[0] = C;
+    __syncthreads();
+    return top < 0 ? -1 : G.ibuf[0];
+}
+
+// Few elements per thread: one per iteration (the four-element code below
+// pays for its empty places: on 2^18 draws of 33 weights at warp width it takes
+// 121 us instead of 93).
+template <int K>
+__device__ int draw_dprs_few(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
+    const int j = G.tid, lane = j & 31, wp = j >> 5;
+    float wB = 0.0f;
+    int C = -1, i = 0;
+    uint4 blk = make_uint4(0, 0, 0, 0);
+#pragma unroll 1
+    for (uint32_t b = 0; b < n; b += K, ++i) {
+        const float wl = b + j < n ? __ldg(w + b + j) : 0.0f;
+        float S = warp_incl_scan(wl, lane), tot;
+        if (K == 32) {
+            tot = __shfl_sync(FULL, S, 31);
+        } else {
+            float* f = G.fbuf + (i & 1) * 32;
+            if (lane == 31) f[wp] = S;
+            __syncthreads();
+            float before = 0.0f;
+            tot = 0.0f;
+#pragma unroll
+            for (int k = 0; k < K / 32; ++k) {
+                const float fk = f[k];
+                if (k == wp) S += before;
+                if (k == K / 32 - 1) tot = fk + before;
+                before += fk;
+            }
+        }
+        if ((i & 3) == 0) blk = elem_block(seed, r, (uint32_t)j, (uint32_t)i >> 2);
+        if (wl > 0.0f && unit24(pick_word(blk, i)) < wl / (S + wB)) C = (int)(b + j);
+        wB += tot;
+    }
+    return G.max_int(C);
+}
+
+template <int K>
+__device__ int draw_zprs_few(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
+    const int j = G.tid;
+    float s = 0.0f;
+    for (uint32_t e = j; e < n; e += K) s += __ldg(w + e);
+    float P = group_scan<K>(G, s) - s;  // exclusive
+    int C = -1, i = 0;
+    uint4 blk = make_uint4(0, 0, 0, 0);
+#pragma unroll 1
+    for (uint32_t e = j; e < n; e += K, ++i) {
+        const float we = __ldg(w + e);
+        P += we;
+        if ((i & 3) == 0) blk = elem_block(seed, r, (uint32_t)j, (uint32_t)i >> 2);
+        if (we > 0.0f && unit24(pick_word(blk, i)) < we / P) C = (int)e;
+    }
+    return zprs_winner(G, C);
+}
+
 // DPRS (Alg. 3): per iteration, k consecutive weights, their inclusive
 // prefix sum plus the weight of the earlier iterations (w_B), one uniform per
-// element against w / (W_P + w_B), and the largest selected index so far.
+// element against w / (W_P + w_B); the largest selected index wins.  Four
+// iterations share a Philox block: their scans run side by side (and, at CTA
+// width, through one barrier), and the maximum is taken once, at the end (a
+// thread's later index is always the larger).
 template <int K>
-__device__ int draw_dprs(Group<K>& G, const float* __restrict__ w, int64_t n, uint64_t seed, uint64_t r) {
-    const int j = G.tid;
+__device__ int draw_dprs(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
+    const int j = G.tid, lane = j & 31, wp = j >> 5;
     float wB = 0.0f;
-    int C = -1, selected = -1;
-    uint4 blk = make_uint4(0, 0, 0, 0);
-    const int64_t iters = (n + K - 1) / K;
-    for (int64_t i = 0; i < iters; ++i) {
-        const int64_t e = j + i * K;
-        const float wl = e < n ? __ldg(w + e) : 0.0f;
-        const float incl = G.incl_scan(wl);
-        if ((i & 3) == 0) blk = elem_block(seed, r, (uint32_t)j, (uint32_t)(i >> 2));
-        const float u = unit24(pick_word(blk, (int)(i & 3)));
-        if (wl > 0.0f && u < wl / (incl + wB)) C = (int)e;
-        selected = G.max_int(C);  // the algorithm reduces every iteration
-        wB += G.total(incl);
+    int C = -1;
+    int half = 0;
+#pragma unroll 1
+    for (uint32_t b = 0; b < n; b += 4 * K) {
+        const uint4 blk = elem_block(seed, r, (uint32_t)j, b / (4 * K));
+        float wl[4], S[4], tot[4];
+        load4<K>(w, n, b, (uint32_t)j, wl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            S[q] = 0.0f;
+            tot[q] = 0.0f;
+            if (b + q * K < n) S[q] = warp_incl_scan(wl[q], lane);
+        }
+        if (K == 32) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) tot[q] = __shfl_sync(FULL, S[q], 31);
+        } else {
+            float* f = G.fbuf + half * 32;
+            half ^= 1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (lane == 31) f[q * 8 + wp] = S[q];
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (b + q * K >= n) break;
+                float before = 0.0f;
+#pragma unroll
+                for (int i = 0; i < K / 32; ++i) {
+                    const float fi = f[q * 8 + i];
+                    if (i == wp) S[q] += before;
+                    if (i == K / 32 - 1) tot[q] = fi + before;
+                    before += fi;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            S[q] += wB;
+            wB += tot[q];
+        }
+        const unsigned m = picks(blk, wl, S);
+        if (m) C = (int)(b + (31 - __clz((int)m)) * K + j);
     }
-    return selected;
+    return G.max_int(C);
 }
 
 // ZPRS (Alg. 4): thread j sums its strided subsequence S_j, an exclusive
 // prefix sum over the threads starts each running total, a second pass tests
 // each element against w / (running total), and the selection of the highest
-// thread that selected anything wins.
+// thread that selected anything wins.  Both passes take four elements at a
+// time, whose loads overlap; the second one's share a Philox block.
 template <int K>
-__device__ int draw_zprs(Group<K>& G, const float* __restrict__ w, int64_t n, uint64_t seed, uint64_t r) {
+__device__ int draw_zprs(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
     const int j = G.tid;
     float s = 0.0f;
-    for (int64_t e = j; e < n; e += K) s += __ldg(w + e);
-    float P = G.incl_scan(s) - s;  // exclusive
-    int C = -1;
-    uint4 blk = make_uint4(0, 0, 0, 0);
-    int64_t i = 0;
-    for (int64_t e = j; e < n; e += K, ++i) {
-        const float we = __ldg(w + e);
-        P += we;
-        if ((i & 3) == 0) blk = elem_block(seed, r, (uint32_t)j, (uint32_t)(i >> 2));
-        const float u = unit24(pick_word(blk, (int)(i & 3)));
-        if (we > 0.0f && u < we / P) C = (int)e;
+#pragma unroll 2
+    for (uint32_t b = 0; b < n; b += 4 * K) {
+        float v[4];
+        load4<K>(w, n, b, (uint32_t)j, v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s += v[q];
     }
-    const int top = G.max_int(C >= 0 ? j : -1);
-    // broadcast the winner's C (K <= 256: through the group's int buffer)
-    if (K == 32) return top < 0 ? -1 : __shfl_sync(FULL, C, top);
-    if (j == top) G.ibuf[0] = C;
-    __syncthreads();
-    const int sel = top < 0 ? -1 : G.ibuf[0];
-    __syncthreads();
-    return sel;
+    float P = group_scan<K>(G, s) - s;  // exclusive
+    int C = -1;
+#pragma unroll 1
+    for (uint32_t b = 0; b < n; b += 4 * K) {
+        const uint4 blk = elem_block(seed, r, (uint32_t)j, b / (4 * K));
+        float v[4], S[4];
+        load4<K>(w, n, b, (uint32_t)j, v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) S[q] = P += v[q];
+        const unsigned m = picks(blk, v, S);
+        if (m) C = (int)(b + (31 - __clz((int)m)) * K + j);
+    }
+    return zprs_winner(G, C);
 }
 
 // The engine's sampler: a warp's exponential race with exponential jumps
-// over 128-entry chunks (prefix sum per chunk, a record only when the skip
-// budget runs out), X kept as an FP32 two-sum; at CTA width each warp takes a
+// over 128-entry chunks (a sum per chunk, a record only when the skip budget
+// runs out), X kept as an FP32 two-sum; at CTA width each warp takes a
 // contiguous segment with its own random stream and the smallest race time
-// wins (ties: smaller index).
+// wins (ties: smaller index).  Record i uses block i of the stream; lane l
+// holds the draws of record have - 32 + l, handed out by shuffles.
 struct Race {
     float tau, Xh, Xl;
     int sel;
-    uint32_t ctr;
+    uint32_t i, have;
+    float u1, nl2;  // this lane's draws: u1 and -log u2
 };
 
-__device__ __noinline__ Race race_record(Race R, int idx, float wv, uint64_t seed, uint64_t r, uint32_t stream) {
-    const uint4 o = philox4x32_10(make_uint4((uint32_t)r, (uint32_t)(r >> 32), 0x80000000u | stream, R.ctr++),
-                                  make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
-    const float u1 = unit_open23(o.x), u2 = unit_open23(o.y);
-    float e;
-    if (isinf(R.tau)) e = -logf(u1);
-    else e = -log1pf(u1 * expm1f(-wv * R.tau));
-    R.tau = e / wv;
-    R.sel = idx;
-    R.Xh = -logf(u2) / R.tau;
-    R.Xl = 0.0f;
-    return R;
+// One chunk, at `base`: the skip budget past it, with every record inside it,
+// in visiting order; wv: this lane's weights, own: their sum.
+__device__ __forceinline__ void race_chunk(Race& R, const float (&wv)[4], float own, int64_t base, int lane,
+                                           uint64_t seed, uint64_t r, uint32_t stream) {
+    const float incl = warp_incl_scan(own, lane);
+    const float tot = __shfl_sync(FULL, incl, 31);
+    if (R.Xh - tot + R.Xl > 0.0f) {
+        const float sh = R.Xh - tot;
+        R.Xl += (R.Xh - sh) - tot;
+        R.Xh = sh;
+        return;
+    }
+    float cum[4];
+    cum[0] = (incl - own) + wv[0];
+#pragma unroll
+    for (int q = 1; q < 4; ++q) cum[q] = cum[q - 1] + wv[q];
+    float target = R.Xh + R.Xl;
+    int last = -1;
+#pragma unroll 1
+    for (;;) {
+        int jj = -1;
+#pragma unroll
+        for (int q = 3; q >= 0; --q)
+            if (lane * 4 + q > last && wv[q] > 0.0f && cum[q] >= target) jj = q;
+        const unsigned m = __ballot_sync(FULL, jj >= 0);
+        if (!m) {
+            R.Xh = target - tot;
+            R.Xl = 0.0f;
+            return;
+        }
+        const int L = __ffs(m) - 1;
+        const float wj = jj >= 2 ? (jj == 3 ? wv[3] : wv[2]) : (jj == 1 ? wv[1] : wv[0]);
+        const float cj = jj >= 2 ? (jj == 3 ? cum[3] : cum[2]) : (jj == 1 ? cum[1] : cum[0]);
+        const float wr = __shfl_sync(FULL, wj, L);
+        const float cr = __shfl_sync(FULL, cj, L);
+        last = L * 4 + __shfl_sync(FULL, jj, L);
+        if (R.i == R.have) {
+            const uint4 o = philox4x32_10(make_uint4((uint32_t)r, (uint32_t)(r >> 32), 0x80000000u | stream, R.i + lane),
+                                          make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+            R.u1 = unit_open23(o.x);
+            R.nl2 = -logf(unit_open23(o.y));
+            R.have += 32;
+        }
+        const float u1 = __shfl_sync(FULL, R.u1, R.i), nl = __shfl_sync(FULL, R.nl2, R.i);
+        ++R.i;
+        float e;
+        if (isinf(R.tau)) e = -logf(u1);
+        else e = -log1pf(u1 * expm1f(-wr * R.tau));
+        R.tau = e / wr;
+        R.sel = (int)(base + last);
+        R.Xh = nl / R.tau;
+        target = cr + R.Xh;
+    }
 }
 
+// Past the first records, four chunks at a time: a chunk's total is the sum
+// that its scan leaves in lane 31, here by an xor butterfly (the same pairs in
+// the same order); the four butterflies share all but their first two steps.
+// vec: w is 16-byte aligned.
 __device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, int lane, uint64_t seed, uint64_t r,
-                             uint32_t stream) {
+                             uint32_t stream, bool vec) {
     Race R;
     R.tau = __int_as_float(0x7f800000);
     R.Xh = 0.0f;
     R.Xl = 0.0f;
     R.sel = -1;
-    R.ctr = 0;
-    for (int64_t base = a; base < b; base += 128) {
-        float wv[4];
+    R.i = 0;
+    R.have = 0;
+    int64_t base = a;
+    while (base < b) {
+        if (R.i && base + 512 <= b) {
+            float own[4], wv[4][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int64_t e = base + lane * 4 + q;
-            wv[q] = e < b ? __ldg(w + e) : 0.0f;
-        }
-        const float own = (wv[0] + wv[1]) + (wv[2] + wv[3]);
-        float incl = own;
+            for (int c = 0; c < 4; ++c) {
+                const float* p = w + base + c * 128 + lane * 4;
+                if (vec) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+                    wv[c][0] = v.x; wv[c][1] = v.y; wv[c][2] = v.z; wv[c][3] = v.w;
+                } else {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float nb = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += nb;
-        }
-        const float tot = __shfl_sync(FULL, incl, 31);
-        if (R.Xh - tot + R.Xl > 0.0f) {
-            const float sh = R.Xh - tot;
-            R.Xl += (R.Xh - sh) - tot;
-            R.Xh = sh;
-            continue;
-        }
-        float cum[4];
-        cum[0] = (incl - own) + wv[0];
-#pragma unroll
-        for (int q = 1; q < 4; ++q) cum[q] = cum[q - 1] + wv[q];
-        float target = R.Xh + R.Xl;
-        int last = -1;
-        for (;;) {
-            int jj = -1;
-#pragma unroll
-            for (int q = 3; q >= 0; --q)
-                if (lane * 4 + q > last && wv[q] > 0.0f && cum[q] >= target) jj = q;
-            const unsigned m = __ballot_sync(FULL, jj >= 0);
-            if (!m) {
-                R.Xh = target - tot;
-                R.Xl = 0.0f;
-                break;
-            }
-            const int L = __ffs(m) - 1;
-            float wj = 0.0f, cj = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q == jj) {
-                    wj = wv[q];
-                    cj = cum[q];
+                    for (int q = 0; q < 4; ++q) wv[c][q] = __ldg(p + q);
                 }
-            const float wr = __shfl_sync(FULL, wj, L);
-            const float cr = __shfl_sync(FULL, cj, L);
-            const int jl = __shfl_sync(FULL, jj, L);
-            last = L * 4 + jl;
-            R = race_record(R, (int)(base + last), wr, seed, r, stream);
-            target = cr + R.Xh;
+                own[c] = (wv[c][0] + wv[c][1]) + (wv[c][2] + wv[c][3]);
+            }
+            const bool b0 = lane & 1, b1 = lane & 2;
+            float v0 = b0 ? own[1] : own[0], v1 = b0 ? own[3] : own[2];
+            v0 += __shfl_xor_sync(FULL, b0 ? own[0] : own[1], 1);
+            v1 += __shfl_xor_sync(FULL, b0 ? own[2] : own[3], 1);
+            float v = b1 ? v1 : v0;
+            v += __shfl_xor_sync(FULL, b1 ? v0 : v1, 2);
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(FULL, v, o);
+            float Xh = R.Xh, Xl = R.Xl;
+            bool ok = true;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float tot = __shfl_sync(FULL, v, c);
+                ok = ok && Xh - tot + Xl > 0.0f;
+                const float sh = Xh - tot;
+                Xl += (Xh - sh) - tot;
+                Xh = sh;
+            }
+            if (ok) {  // no record in any of them (the common case)
+                R.Xh = Xh;
+                R.Xl = Xl;
+                base += 512;
+                continue;
+            }
+        }
+        // chunk by chunk: the first ones of a segment, its end, and the four
+        // around a record
+        const int64_t stop = R.i ? min(b, base + 512) : min(b, base + 128);
+#pragma unroll 1
+        for (; base < stop; base += 128) {
+            float wv[4];
+            const int64_t e = base + lane * 4;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) wv[q] = e + q < b ? __ldg(w + e + q) : 0.0f;
+            race_chunk(R, wv, (wv[0] + wv[1]) + (wv[2] + wv[3]), base, lane, seed, r, stream);
         }
     }
     return R;
@@ -238,12 +433,13 @@ __device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, 
 template <int K>
 __device__ int draw_expj(Group<K>& G, const float* __restrict__ w, int64_t n, uint64_t seed, uint64_t r) {
     const int lane = G.tid & 31;
-    if (K == 32) return race_segment(w, 0, n, lane, seed, r, 0).sel;
+    const bool vec = ((uintptr_t)w & 15) == 0;
+    if (K == 32) return race_segment(w, 0, n, lane, seed, r, 0, vec).sel;
     // CTA width: K / 32 contiguous segments (multiples of 128 entries)
     const int wp = G.tid >> 5;
     const int64_t seg = ((n + K / 32 - 1) / (K / 32) + 127) / 128 * 128;
     const int64_t a = min(n, (int64_t)wp * seg), b = min(n, a + seg);
-    const Race R = race_segment(w, a, b, lane, seed, r, (uint32_t)wp);
+    const Race R = race_segment(w, a, b, lane, seed, r, (uint32_t)wp, vec);
     __shared__ unsigned long long best;
     if (G.tid == 0) best = ~0ull;
     __syncthreads();
@@ -255,9 +451,9 @@ __device__ int draw_expj(Group<K>& G, const float* __restrict__ w, int64_t n, ui
 }
 
 template <int METHOD, int K>
-__global__ void __launch_bounds__(256) sampler_kernel(const float* __restrict__ w, int64_t n, int64_t reps,
+__global__ void __launch_bounds__(256, METHOD == SAMP_EXPJ ? 5 : 8) sampler_kernel(const float* __restrict__ w, int64_t n, int64_t reps,
                                                       uint64_t seed, int32_t* __restrict__ out) {
-    __shared__ float fbuf[8];
+    __shared__ float fbuf[64];
     __shared__ int ibuf[8];
     Group<K> G;
     G.fbuf = fbuf;
@@ -267,9 +463,16 @@ __global__ void __launch_bounds__(256) sampler_kernel(const float* __restrict__ 
     const int gi = (int)(threadIdx.x / K);
     for (int64_t r = (int64_t)blockIdx.x * groups + gi; r < reps; r += (int64_t)gridDim.x * groups) {
         int sel;
-        if (METHOD == SAMP_DPRS) sel = draw_dprs<K>(G, w, n, seed, (uint64_t)r);
-        else if (METHOD == SAMP_ZPRS) sel = draw_zprs<K>(G, w, n, seed, (uint64_t)r);
-        else sel = draw_expj<K>(G, w, n, seed, (uint64_t)r);
+        // (the lines between the three lie where they measured equal)
+        constexpr int64_t kFew = K == 32 ? 256 : 768;
+        if (METHOD == SAMP_EXPJ) sel = draw_expj<K>(G, w, n, seed, (uint64_t)r);
+        else if (n <= K) sel = draw_short<K, METHOD == SAMP_ZPRS>(G, w, (uint32_t)n, seed, (uint64_t)r);
+        else if (METHOD == SAMP_DPRS)
+            sel = n <= kFew ? draw_dprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
+                            : draw_dprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
+        else
+            sel = n <= kFew ? draw_zprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
+                            : draw_zprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
         if (G.tid == 0) out[r] = sel;
     }
 }
