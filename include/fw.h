@@ -112,7 +112,11 @@ typedef struct {
  *   slots           walks resident per CTA: the local task pool P_L, at most
  *                   8 per warp (default 4 per warp).
  *   d_warp          degree threshold d_t: rows with d <= d_warp are sampled
- *                   by one warp, larger rows by the whole CTA (default 65536).
+ *                   by one warp, larger rows by the whole CTA (default 65536;
+ *                   while it is not set, a batch launch also shares rows above
+ *                   16384 entries, in small exact launches above 4096, once a
+ *                   warp of the CTA has no walk left, and in fast mode it
+ *                   shares no others).
  *   ctas_per_sm     persistent CTAs per SM (0 = as many as fit).
  * Zero fields mean "default".  No field changes a walk's result: exact mode is
  * bit-identical to the CPU oracle under every tuning, and fast mode draws each

@@ -814,6 +814,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // fetch the next row's offsets, and hand the slot back (READY or FINISH).
 // `hub`: the slot may belong to another warp, so the offsets must have landed
 // first.
+template <bool PPR>
 __device__ __forceinline__ void commit(const GraphDev& g, Slot& s, int sel, bool hub) {
     const ReqDev& R = s.rq;
     const long long beg = s.row[0];
@@ -822,7 +823,7 @@ __device__ __forceinline__ void commit(const GraphDev& g, Slot& s, int sel, bool
     fetch_row(g, s, next);
     const int t = s.t;
     bool stop = false;
-    if (R.algo == FW_PPR) stop = step_block(R.seed, (uint64_t)(R.q_id0 + s.q), (uint32_t)t).z < R.t_stop;
+    if (PPR && R.algo == FW_PPR) stop = step_block(R.seed, (uint64_t)(R.q_id0 + s.q), (uint32_t)t).z < R.t_stop;
     const int k = s.k;
     R.paths[s.q * ((long long)R.max_len + 1) + k] = next;
     s.k = k + 1;
@@ -876,6 +877,7 @@ struct Launch {
     long long total;
     unsigned long long* cursor;
     unsigned long long* counters;
+    int d_always;   // rows above it are hub tasks whether or not the CTA has a warp without walks
     int claimers;   // warps of a CTA that claim queries (the others only help with hub tasks)
     int seg_q;      // exact mode: quads per hub segment
     unsigned nap;   // sleep of a warp that has no walk left between looks for hub work (ns); 0: it returns
@@ -994,8 +996,12 @@ __device__ __noinline__ void retire_walk(const ServeDev& sv, Slot& sl, unsigned 
 
 // Publish the step of slot sl as a CTA hub task of nseg segments, if a task
 // entry is free; if none is, the walk stays ready and is published on a later
-// visit, after this warp has helped the open tasks.  Warp-collective.
-__device__ __noinline__ void hub_publish(CtaHead& head, WarpHead& wh, Slot& sl, int slot, int nseg, int lane) {
+// visit, after this warp has helped the open tasks.  False if the row is not
+// worth it: no warp of the CTA is without walks of its own (and `always` does
+// not ask for it).  Warp-collective.
+__device__ __noinline__ bool hub_publish(CtaHead& head, WarpHead& wh, Slot& sl, int slot, bool always, int nseg,
+                                         int lane) {
+    if (!always && !__shfl_sync(FULL, *(volatile int*)&head.working < (int)(blockDim.x >> 5), 0)) return false;
     int ok = 0;
     if (lane == 0) {
 #pragma unroll 1
@@ -1022,6 +1028,7 @@ __device__ __noinline__ void hub_publish(CtaHead& head, WarpHead& wh, Slot& sl, 
         if (lane == 0) wh.nap = min(nap * 2u, 1024u);
         __syncwarp();
     }
+    return true;
 }
 
 // The walk to advance when the next one in turn is not ready: refills empty
@@ -1109,8 +1116,9 @@ __device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restric
     return PICK_AGAIN;
 }
 
-// N2V, LAB: the launch may hold node2vec / MetaPath requests (a build without
-// them is smaller: see the instruction cache above).
+// N2V, LAB: the launch may hold node2vec / MetaPath requests; with N2V, PPR
+// requests need LAB too (a build without them is smaller: see the instruction
+// cache above).
 // SERVE: the served form's build (queries claimed from the request ring,
 // completion stamps, idle polling); the batch build compiles all of that out.
 template <bool EXACT, bool N2V, bool LAB, bool SERVE>
@@ -1181,8 +1189,7 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
             stream = seg & 0xFF;
             ra += stream * sq;
             lim = min(lim, ra + sq);
-        } else if (lim > d_t) {
-            hub_publish(head, wh, sl, s, (lim - ra + sq - 1) / sq, lane);
+        } else if (lim > d_t && hub_publish(head, wh, sl, s, lim > L.d_always, (lim - ra + sq - 1) / sq, lane)) {
             continue;
         }
 
@@ -1303,7 +1310,7 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
                 *(volatile int*)&sl.state = ST_FINISH;  // nothing selectable (or a dead end): the walk stops here
             } else {
                 count_step(wh.cnt, (int)(sl.row[1] - sl.row[0]), sl.rq.algo, seg >= 0);
-                commit(g, sl, sel, seg >= 0);
+                commit<LAB || !N2V>(g, sl, sel, seg >= 0);
             }
             if (seg >= 0) {
                 __threadfence_block();

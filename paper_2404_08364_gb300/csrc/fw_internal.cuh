@@ -18,8 +18,9 @@ namespace fw {
 // generator state lives anywhere (the paper keeps cuRAND states in shared
 // memory, Section 4.3; a counter-based generator needs none).
 // ---------------------------------------------------------------------------
-__host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
-#pragma unroll
+template <int UNROLL>
+__host__ __device__ __forceinline__ uint4 philox4x32_10_by(uint4 c, uint2 k) {
+#pragma unroll UNROLL
     for (int r = 0; r < 10; ++r) {
         if (r) {
             k.x += 0x9E3779B9u;
@@ -34,11 +35,15 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
     return c;
 }
 
+__host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) { return philox4x32_10_by<10>(c, k); }
+
 // Per-step block: counter (t, q_lo, q_hi, 0), key (seed_lo, seed_hi).
 // Words x|y<<32 give the exact-mode 64-bit draw, word z the PPR stop test.
 __host__ __device__ __forceinline__ uint4 step_block(uint64_t seed, uint64_t qid, uint32_t t) {
-    return philox4x32_10(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32), 0u),
-                         make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+    // (rolled here and below: the walk engine evaluates one block per step and
+    // its loop has to fit the instruction cache)
+    return philox4x32_10_by<1>(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32), 0u),
+                               make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
 }
 
 // Fast-mode reservoir draws: counter word 3 = 0x80000000 | lane << 16 | k.
@@ -47,9 +52,9 @@ __host__ __device__ __forceinline__ uint4 step_block(uint64_t seed, uint64_t qid
 // the per-step block.
 __device__ __forceinline__ uint4 lane_block(uint64_t seed, uint64_t qid, uint32_t t, uint32_t lane,
                                             uint32_t k) {
-    return philox4x32_10(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32),
-                                    0x80000000u | ((lane & 0x7FFFu) << 16) | (k & 0xFFFFu)),
-                         make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+    return philox4x32_10_by<1>(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32),
+                                          0x80000000u | ((lane & 0x7FFFu) << 16) | (k & 0xFFFFu)),
+                               make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
 }
 
 // ---------------------------------------------------------------------------

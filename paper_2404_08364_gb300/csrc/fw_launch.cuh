@@ -41,8 +41,17 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
     if (e != cudaSuccess) return e;
     const int64_t resident = (int64_t)sms * per_sm * (threads / 32);
     int64_t grid = (int64_t)sms * per_sm;
-    Launch L = {reqs.ext, n_req, (long long)total, cursor, counters, threads / 32, kSegQuads, 4096u};
+    Launch L = {reqs.ext, n_req, (long long)total, cursor, counters, tu.d_warp, threads / 32, kSegQuads, 4096u};
     int d_t = tu.d_warp;
+    if (!tu.own_d) {
+        // Sharing a row costs throughput (hand-offs, fresh N(prev) cursors,
+        // waiting owners) and gains latency: unless the caller set d_t, rows
+        // from one segment on are shared while the CTA has a warp without walks
+        // of its own.  Fast mode does not share otherwise (PPR from the
+        // R-MAT-22 hub: 4.7 -> 4.1 ms); exact mode does above the default d_t.
+        d_t = 4 * kSegQuads;
+        if (!EXACT) L.d_always = 1 << 30;
+    }
     if (total < resident) {
         // Fewer walks than resident warps: latency counts.  One walk per warp
         // (a warp advances its walks one after another), spread evenly over
@@ -54,9 +63,9 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
         // fast 868 -> 777, exact 1,095 -> 712 (helpers); 129 PPR walks on
         // R-MAT-22 222 -> 201.
         use = 1;
-        if (!tu.own_d) {
-            d_t = min(d_t, EXACT ? 4096 : 4 * kSegQuads);
-            if (EXACT) L.seg_q = 512;
+        if (!tu.own_d && EXACT) {
+            d_t = 4096;
+            L.seg_q = 512;
         }
         if (!own && g.d_max > d_t) {
             threads = 768;
@@ -80,7 +89,8 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
 template <bool EXACT>
 cudaError_t launch_mode(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                         unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
-    const bool n2v = reqs.algos >> FW_NODE2VEC & 1u, lab = reqs.algos >> FW_METAPATH & 1u;
+    const bool n2v = reqs.algos >> FW_NODE2VEC & 1u;
+    const bool lab = reqs.algos >> FW_METAPATH & 1u || (n2v && reqs.algos >> FW_PPR & 1u);
     return n2v ? (lab ? launch_as<EXACT, true, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
                       : launch_as<EXACT, true, false>(g, reqs, n_req, total, cursor, counters, tu, stream))
                : (lab ? launch_as<EXACT, false, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
@@ -103,7 +113,7 @@ cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, 
     if (e != cudaSuccess) return e;
     ReqTable tab;
     memset(&tab, 0, sizeof tab);
-    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters, warps, kSegQuads, 0u};
+    const Launch L = {nullptr, 0, 0ll, &scratch->cursor, scratch->counters, tu.d_warp, warps, kSegQuads, 0u};
     kern<<<(unsigned)(sms - min(8, sms - 1)), warps * 32, smem, stream>>>(g, tab, L, sw, tu.d_warp, sv);
     return cudaGetLastError();
 }
