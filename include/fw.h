@@ -110,7 +110,8 @@ typedef struct {
  *                   default, 512, which leaves the shape to the engine while
  *                   ctas_per_sm is 0 too).
  *   slots           walks resident per CTA: the local task pool P_L, at most
- *                   8 per warp (default 4 per warp).
+ *                   8 per warp (default, nominally, 4 per warp; while it is
+ *                   not set the engine runs one).
  *   d_warp          degree threshold d_t: rows with d <= d_warp are sampled
  *                   by one warp, larger rows by the whole CTA (default 65536;
  *                   while it is not set, a batch launch also shares rows above

@@ -154,6 +154,7 @@ struct Tuning {
     int slots;
     int d_warp;
     int ctas_per_sm;
+    bool own_slots;  // slots was set by the caller (else one walk per warp)
     bool own_d;      // d_warp was set by the caller
     bool own_shape;  // block_threads was set by the caller (else each engine may take the CTA size that suits it)
 };

@@ -25,11 +25,20 @@ cudaError_t engine_grid(K kern, int threads, size_t smem, const Tuning& tu, int*
     return cudaSuccess;
 }
 
+// One walk per warp unless the caller asked for more: a walk that goes on at once
+// finds the row it came from (node2vec's N(prev)) still in L2, and its slots'
+// shared memory is L1's.  Measured against four walks taken in turn (ms):
+// node2vec R-MAT-25 187.1 -> 182.4, R-MAT-20 35.8 -> 33.1, exact 12.9 -> 10.4,
+// weighted R-MAT-22 15.8 -> 15.0, MetaPath + PPR 7.9 -> 7.3.
+inline int walks_per_warp(const Tuning& tu) {
+    return tu.own_slots ? max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32))) : 1;
+}
+
 template <bool EXACT, bool N2V, bool LAB>
 cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                       unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
     auto kern = walk_kernel<EXACT, N2V, LAB, false>;
-    const int sw = max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
+    const int sw = walks_per_warp(tu);
     // CTAs of 256 threads unless the caller chose: at 80 registers three of
     // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
     // (R-MAT-25 node2vec: 240 -> 202 ms), and a hub row's last segments hold
@@ -106,7 +115,7 @@ cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, 
     // and through the hardware queues streams share, the server's own copies
     // queued behind them.
     const int warps = 24;
-    const int sw = max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
+    const int sw = walks_per_warp(tu);
     const size_t smem = cta_smem<EXACT, true>(warps, sw);
     int sms = 0, per_sm = 0;
     cudaError_t e = engine_grid(kern, warps * 32, smem, tu, &sms, &per_sm);

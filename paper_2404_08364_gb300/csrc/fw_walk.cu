@@ -3,7 +3,7 @@
 
 namespace fw {
 
-Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false, false}; }
+Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false, false, false}; }
 
 Tuning sanitize_tuning(Tuning t) {
     const Tuning d = default_tuning();
@@ -11,7 +11,10 @@ Tuning sanitize_tuning(Tuning t) {
         t.block_threads = d.block_threads;
         t.own_shape = false;
     }
-    if (t.slots <= 0) t.slots = 4 * (t.block_threads / 32);  // four walks per warp
+    if (t.slots <= 0) {
+        t.slots = 4 * (t.block_threads / 32);  // (nominal)
+        t.own_slots = false;
+    }
     if (t.slots > (t.block_threads / 32) * kSlotsPerWarp) t.slots = (t.block_threads / 32) * kSlotsPerWarp;
     if (t.d_warp <= 0) {
         t.d_warp = d.d_warp;
