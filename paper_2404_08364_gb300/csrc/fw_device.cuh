@@ -77,6 +77,27 @@ __device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
+// Read-only loads under a predicate, as single instructions: the compiler
+// neither turns them into branches, one waiting for the other, nor moves them
+// down past later volatile ones to where their value is used.
+__device__ __forceinline__ int ldg_if(const int32_t* p, bool ok, int other) {
+    int v;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\tmov.b32 %0, %3;\n\t@q ld.global.nc.b32 %0, [%1];\n\t}"
+        : "=&r"(v)
+        : "l"(p), "r"((int)ok), "r"(other));
+    return v;
+}
+__device__ __forceinline__ float4 ldg_if(const float4* p, bool ok) {
+    float4 v;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %5, 0;\n\tmov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\t"
+        "mov.b32 %3, 0;\n\t@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+        : "=&f"(v.x), "=&f"(v.y), "=&f"(v.z), "=&f"(v.w)
+        : "l"(p), "r"((int)ok));
+    return v;
+}
+
 // Orders this thread's ordinary shared-memory stores before later bulk copies
 // into the same bytes.
 __device__ __forceinline__ void fence_proxy_async_cta() {

@@ -104,7 +104,8 @@ struct CtaHead {
 };
 
 // Per-warp shared memory.
-struct WarpHead {
+struct __align__(16) WarpHead {
+    float rec[16];                  // a lane's eight running sums and weights (stage_records)
     unsigned long long cnt[C_NUM];
     unsigned long long idle_since;  // when the warp ran out of work (0: it has some)
     unsigned nap;                   // idle back-off (ns)
@@ -112,7 +113,7 @@ struct WarpHead {
     int done;                       // no walk is left either (not counted in CtaHead::working)
 };
 constexpr int kHeadBytes = (sizeof(CtaHead) + 127) & ~127;
-constexpr int kWarpHeadBytes = (sizeof(WarpHead) + 127) & ~127;
+constexpr int kWarpHeadBytes = (sizeof(WarpHead) + 63) & ~63;
 
 // Offsets inside a warp's area.  node2vec: a chunk's columns (and one word
 // that equals no vertex id), its membership bytes, the splitters of a dense
@@ -123,7 +124,7 @@ struct Area {
     static constexpr int MASK = COL + (N2V ? CHUNK * 4 + 16 : 0);
     static constexpr int SPL = MASK + (N2V ? CHUNK : 0);
     static constexpr int BAR = SPL + (N2V ? kSplCap * 4 : 0);
-    static constexpr int HEAD = (BAR + (N2V ? 8 : 0) + 127) & ~127;
+    static constexpr int HEAD = (BAR + (N2V ? 8 : 0) + 63) & ~63;
     static constexpr int BYTES = HEAD + kWarpHeadBytes;
 };
 
@@ -188,8 +189,9 @@ __device__ __forceinline__ int seg_entries(int r_a, int d, int seg_q) {
 // budget past the stage.  The stage starts at row index e0; w: this lane's
 // entries (0: outside the row or excluded), row indices e0 + 4 lane + j
 // (j < 4) and e0 + 4 lane + 124 + j (j >= 4); own: their sum.
+template <bool N2V>
 __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float own, int e0, int lane,
-                                              const Slot& sl, int stream) {
+                                              float* __restrict__ rec, const Slot& sl, int stream) {
     float incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -202,38 +204,69 @@ __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float
     cum[0] = (incl - own) + w[0];
 #pragma unroll
     for (int j = 1; j < 8; ++j) cum[j] = cum[j - 1] + w[j];
-    unsigned live = 0;  // entries that a record may still fall on
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (w[j] > 0.0f) live |= 1u << j;
     float target = R.Xh + R.Xl;  // a record falls on the first entry whose cumulative weight reaches target
+    unsigned live = 0;           // N2V: entries that a record may still fall on
+    int last = -1, from = 0;     // else: visiting position of the last record, first lane that may hold the next
+    if (N2V) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (w[j] > 0.0f) live |= 1u << j;
+    }
 #pragma unroll 1
     for (;;) {
-        // this lane's first entry that reaches target: a binary search of cum
-        int j = cum[3] < target ? 4 : 0;
-        j += (j ? cum[5] : cum[1]) < target ? 2 : 0;
-        j += (j & 4 ? (j & 2 ? cum[6] : cum[4]) : (j & 2 ? cum[2] : cum[0])) < target ? 1 : 0;
-        // (j = 7 stands for 7 and for none)
-        unsigned hit = live >> j << j;
-        if (cum[7] < target) hit = 0u;
-        const unsigned m = __ballot_sync(FULL, hit != 0u);
-        if (!m) {
-            R.Xh = target - tot;
-            R.Xl = 0.0f;
-            return;
+        int L, jj;
+        float wr, cr;  // the record's weight and running sum
+        if (N2V) {
+            // this lane's first entry that reaches target: a binary search of cum
+            int j = cum[3] < target ? 4 : 0;
+            j += (j ? cum[5] : cum[1]) < target ? 2 : 0;
+            j += (j & 4 ? (j & 2 ? cum[6] : cum[4]) : (j & 2 ? cum[2] : cum[0])) < target ? 1 : 0;
+            // (j = 7 stands for 7 and for none)
+            unsigned hit = live >> j << j;
+            if (cum[7] < target) hit = 0u;
+            const unsigned m = __ballot_sync(FULL, hit != 0u);
+            if (!m) break;
+            L = __ffs(m) - 1;
+            jj = __shfl_sync(FULL, __ffs(hit) - 1, L);
+            const bool b0 = jj & 1, b1 = jj & 2, b2 = jj & 4;
+            wr = b2 ? (b1 ? (b0 ? w[7] : w[6]) : (b0 ? w[5] : w[4])) : (b1 ? (b0 ? w[3] : w[2]) : (b0 ? w[1] : w[0]));
+            cr = b2 ? (b1 ? (b0 ? cum[7] : cum[6]) : (b0 ? cum[5] : cum[4]))
+                    : (b1 ? (b0 ? cum[3] : cum[2]) : (b0 ? cum[1] : cum[0]));
+            wr = __shfl_sync(FULL, wr, L);
+            cr = __shfl_sync(FULL, cr, L);
+            // later records lie beyond this one
+            if (lane < L) live = 0u;
+            if (lane == L) live = live >> (jj + 1) << (jj + 1);
+        } else {
+            // The first lane whose entries reach target hands them out through
+            // shared memory and eight lanes look at one each: fewer
+            // instructions than the search and the selects above (weighted
+            // R-MAT-22 14.8 -> 14.5 ms).  In the node2vec build it measured
+            // slower (R-MAT-25 182 -> 191 ms: the barrier keeps the compiler
+            // from moving loads ahead).
+            const unsigned m = from > 31 ? 0u : __ballot_sync(FULL, cum[7] >= target && own > 0.0f) >> from << from;
+            if (!m) break;
+            L = __ffs(m) - 1;
+            if (lane == L) {
+                reinterpret_cast<float4*>(rec)[0] = make_float4(cum[0], cum[1], cum[2], cum[3]);
+                reinterpret_cast<float4*>(rec)[1] = make_float4(cum[4], cum[5], cum[6], cum[7]);
+                reinterpret_cast<float4*>(rec)[2] = make_float4(w[0], w[1], w[2], w[3]);
+                reinterpret_cast<float4*>(rec)[3] = make_float4(w[4], w[5], w[6], w[7]);
+            }
+            __syncwarp();
+            const float c = rec[lane & 7], x = rec[8 + (lane & 7)];
+            const unsigned in = __ballot_sync(FULL, c >= target && x > 0.0f && 8 * L + (lane & 7) > last) & 0xFFu;
+            if (!in) {  // (only where the last record's own entry still reaches target)
+                from = L + 1;
+                continue;
+            }
+            jj = __ffs(in) - 1;
+            wr = __shfl_sync(FULL, x, jj);
+            cr = __shfl_sync(FULL, c, jj);
+            last = 8 * L + jj;
+            from = L;
         }
-        const int L = __ffs(m) - 1;
-        const int jj = __shfl_sync(FULL, __ffs(hit) - 1, L);
-        const bool b0 = jj & 1, b1 = jj & 2, b2 = jj & 4;
-        const float wj = b2 ? (b1 ? (b0 ? w[7] : w[6]) : (b0 ? w[5] : w[4])) : (b1 ? (b0 ? w[3] : w[2]) : (b0 ? w[1] : w[0]));
-        const float cj = b2 ? (b1 ? (b0 ? cum[7] : cum[6]) : (b0 ? cum[5] : cum[4]))
-                            : (b1 ? (b0 ? cum[3] : cum[2]) : (b0 ? cum[1] : cum[0]));
-        const float wr = __shfl_sync(FULL, wj, L);
-        const float cr = __shfl_sync(FULL, cj, L);
         R.sel = e0 + 4 * L + jj + (jj >= 4 ? 124 : 0);
-        // later records lie beyond this one
-        if (lane < L) live = 0u;
-        if (lane == L) live = live >> (jj + 1) << (jj + 1);
         if (R.i == R.have) {
             const uint4 o = lane_block(sl.rq.seed, (uint64_t)(sl.rq.q_id0 + sl.q), (uint32_t)sl.t, (uint32_t)stream,
                                        (uint32_t)(R.i + lane) >> 1);
@@ -254,6 +287,8 @@ __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float
         R.Xh = __fdividef(nl, R.tau);
         target = cr + R.Xh;
     }
+    R.Xh = target - tot;
+    R.Xl = 0.0f;
 }
 
 // Offer a pair of stages: w[8 h + j] = this lane's entries of stage h, ordered
@@ -261,8 +296,9 @@ __device__ __forceinline__ void stage_records(Res& R, const float (&w)[8], float
 // A stage's total is the xor butterfly sum of its lanes' sums (the same in
 // every lane, as a + b = b + a in IEEE arithmetic); the two butterflies share
 // their last four steps, one stage in each half of the warp.
-__device__ __forceinline__ void offer_pair(Res& R, float (&w)[16], bool two, int e0, int lane, const Slot& sl,
-                                           int stream) {
+template <bool N2V>
+__device__ __forceinline__ void offer_pair(Res& R, float (&w)[16], bool two, int e0, int lane,
+                                           float* __restrict__ rec, const Slot& sl, int stream) {
     const float own0 = ((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]));
     const float own1 = ((w[8] + w[9]) + (w[10] + w[11])) + ((w[12] + w[13]) + (w[14] + w[15]));
     const bool up = lane & 16;
@@ -292,7 +328,7 @@ __device__ __forceinline__ void offer_pair(Res& R, float (&w)[16], bool two, int
             R.Xh = s;
         } else {
             const float ws[8] = {w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]};
-            stage_records(R, ws, own, e0, lane, sl, stream);
+            stage_records<N2V>(R, ws, own, e0, lane, rec, sl, stream);
         }
         if (!two) return;
         two = false;
@@ -446,17 +482,24 @@ __device__ __forceinline__ void load_pair(const float* __restrict__ wrow, const 
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int rel = at + 128 * k;
-            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (rel < lim) {
-                if (rel + 4 <= left) {
-                    v = __ldg(q + 32 * k);
-                    if (LAB && lrow) l[k] = __ldg(ql + 32 * k);
-                } else {
-                    v = load_quad_tail(wrow, rel, left);
+            const bool in = rel < lim && rel + 4 <= left;
+            const float4 v = ldg_if(q + 32 * k, in);
+            if (LAB && lrow) l[k] = ldg_if(ql + 32 * k, in, 0);
+            w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
+        }
+        if (lim + 3 > left) {
+            // a range that ends with the arrays: its last quad may lie across
+            // their end
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int rel = at + 128 * k;
+                if (rel < lim && rel + 4 > left) {
+                    const float4 v = load_quad_tail(wrow, rel, left);
+                    w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
                     if (LAB && lrow) l[k] = load_labels_tail(lrow, rel, left);
                 }
             }
-            w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
+            __syncwarp();
         }
 #pragma unroll
         for (int j = 0; j < 16; ++j)
@@ -521,7 +564,7 @@ __device__ __forceinline__ void load_b128(const int32_t* __restrict__ B, int pd,
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int idx = base + 32 * i + lane;
-        v[i] = idx < pd ? __ldg(B + idx) : INT_BIG;
+        v[i] = ldg_if(B + idx, idx < pd, INT_BIG);
     }
 }
 
@@ -569,18 +612,26 @@ __device__ __noinline__ void dense_members(const int32_t* __restrict__ B, int en
 #pragma unroll 1
         while (more) {
             more = false;
+            int mid[4], v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                mid[j] = (int)(((unsigned)a[j] + (unsigned)b[j]) >> 1);
+                v[j] = ldg_if(B + mid[j], a[j] < b[j], 0);
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (a[j] < b[j]) {
                     more = true;
-                    const int mid = (int)(((unsigned)a[j] + (unsigned)b[j]) >> 1);
-                    if (__ldg(B + mid) < x[j]) a[j] = mid + 1;
-                    else b[j] = mid;
+                    if (v[j] < x[j]) a[j] = mid[j] + 1;
+                    else b[j] = mid[j];
                 }
         }
+        int hit[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) hit[j] = ldg_if(B + a[j], a[j] < end, -1);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (a[j] < end && __ldg(B + a[j]) == x[j]) area[Area<true>::MASK + e0 + 32 * j] = 1;
+            if (a[j] < end && hit[j] == x[j]) area[Area<true>::MASK + e0 + 32 * j] = 1;
     }
     __syncwarp();  // the splitters are rewritten by the next dense chunk
 }
@@ -758,7 +809,7 @@ __device__ __forceinline__ bool scan_range(const GraphDev& g, const Slot& sl, in
                 }
             }
             if (EXACT) exact_pair(X, w, rp, lane);
-            else offer_pair(R, w, rp + STAGE < lim, rp, lane, sl, stream);
+            else offer_pair<N2V>(R, w, rp + STAGE < lim, rp, lane, reinterpret_cast<WarpHead*>(area + Area<N2V>::HEAD)->rec, sl, stream);
         }
         if (N2V) __syncwarp();  // the membership bytes are cleared for the next chunk
     }
