@@ -131,7 +131,8 @@ class ClockSampler:
                 "reasons": sorted(reasons)}
 
 
-KERNEL_SOURCES = ("paper_2404_08364_gb300/csrc/fw_walk.cu", "paper_2404_08364_gb300/csrc/fw_internal.cuh")
+KERNEL_SOURCES = tuple("paper_2404_08364_gb300/csrc/" + f for f in
+                       ("fw_engine.cuh", "fw_device.cuh", "fw_launch.cuh", "fw_fast.cu", "fw_walk.cu", "fw_internal.cuh"))
 
 
 def _code_tokens(text):
