@@ -89,3 +89,24 @@ def test_bad_columns_and_weights_are_found(at):
         r = rp.copy()
         r[k] = v
         assert _status(r, col, w, wu, validate=False) == _fw.FW_EINVAL
+
+
+@pytest.mark.parametrize("drop", [0, 1, 2, 3])
+def test_copied_arrays_walk_as_borrowed_ones(drop):
+    """The arrays of a copied graph lie one behind the other: sizes with every
+    remainder of 4 entries, from host and from device memory."""
+    need_gpu()
+    built()
+    from paper_2404_08364_gb300 import DeviceGraph
+    rp, col, w, wu = _graph()
+    m = col.size - drop
+    rp, col, w, wu = np.minimum(rp, m), col[:m], w[:m], np.arange(1, m + 1, dtype=np.int32)
+    host = [torch.from_numpy(np.ascontiguousarray(x)) for x in (rp, col, w, wu, (np.arange(m) % 3).astype(np.int8))]
+    dev = [x.cuda() for x in host]
+    graphs = [DeviceGraph.from_tensors(*host), DeviceGraph.from_tensors(*dev), DeviceGraph.from_tensors(*dev, borrow=True)]
+    starts = torch.arange(64, dtype=torch.int32).cuda() % 8
+    for algo, mode in (("weighted", "fast"), ("weighted", "exact"), ("metapath", "fast"), ("metapath", "exact")):
+        outs = [g.walk(algo, starts, 6, 5, mode=mode, schema=(0, 1, 2)) for g in graphs]
+        for paths, plen in outs[1:]:
+            assert torch.equal(paths, outs[0][0]) and torch.equal(plen, outs[0][1])
+        assert int(outs[0][1].sum()) > 64  # (some walk moves)
