@@ -153,7 +153,7 @@ __device__ __forceinline__ int zprs_winner(Group<K>& G, int C) {
 
 // Few elements per thread: one per iteration (the four-element code below
 // pays for its empty places: on 2^18 draws of 33 weights at warp width it takes
-// 121 us instead of 93).
+// 121 us instead of 89).
 template <int K>
 __device__ int draw_dprs_few(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
     const int j = G.tid, lane = j & 31, wp = j >> 5;
@@ -271,7 +271,7 @@ template <int K>
 __device__ int draw_zprs(Group<K>& G, const float* __restrict__ w, uint32_t n, uint64_t seed, uint64_t r) {
     const int j = G.tid;
     float s = 0.0f;
-#pragma unroll 2
+#pragma unroll 4
     for (uint32_t b = 0; b < n; b += 4 * K) {
         float v[4];
         load4<K>(w, n, b, (uint32_t)j, v);
@@ -282,9 +282,9 @@ __device__ int draw_zprs(Group<K>& G, const float* __restrict__ w, uint32_t n, u
     int C = -1;
 #pragma unroll 1
     for (uint32_t b = 0; b < n; b += 4 * K) {
-        const uint4 blk = elem_block(seed, r, (uint32_t)j, b / (4 * K));
         float v[4], S[4];
         load4<K>(w, n, b, (uint32_t)j, v);
+        const uint4 blk = elem_block(seed, r, (uint32_t)j, b / (4 * K));
 #pragma unroll
         for (int q = 0; q < 4; ++q) S[q] = P += v[q];
         const unsigned m = picks(blk, v, S);
@@ -361,12 +361,7 @@ __device__ __forceinline__ void race_chunk(Race& R, const float (&wv)[4], float 
     }
 }
 
-// Past the first records, four chunks at a time: a chunk's total is the sum
-// that its scan leaves in lane 31, here by an xor butterfly (the same pairs in
-// the same order); the four butterflies share all but their first two steps.
-// vec: w is 16-byte aligned.
-__device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, int lane, uint64_t seed, uint64_t r,
-                             uint32_t stream, bool vec) {
+__device__ __forceinline__ Race race_start() {
     Race R;
     R.tau = __int_as_float(0x7f800000);
     R.Xh = 0.0f;
@@ -374,6 +369,16 @@ __device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, 
     R.sel = -1;
     R.i = 0;
     R.have = 0;
+    return R;
+}
+
+// Past the first records, four chunks at a time: a chunk's total is the sum
+// that its scan leaves in lane 31, here by an xor butterfly (the same pairs in
+// the same order); the four butterflies share all but their first two steps.
+// vec: w is 16-byte aligned.
+__device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, int lane, uint64_t seed, uint64_t r,
+                             uint32_t stream, bool vec) {
+    Race R = race_start();
     int64_t base = a;
     while (base < b) {
         if (R.i && base + 512 <= b) {
@@ -430,16 +435,30 @@ __device__ Race race_segment(const float* __restrict__ w, int64_t a, int64_t b, 
     return R;
 }
 
-template <int K>
+// A segment of at most one chunk: an own kernel, whose fewer registers leave
+// room for more warps (2^18 draws at warp width, in us: 4 weights 108 against 134,
+// 127 weights 246 against 284; at CTA width 4 weights 290 against 435).
+__device__ Race race_short(const float* __restrict__ w, int a, int b, int lane, uint64_t seed, uint64_t r, uint32_t stream) {
+    Race R = race_start();
+    const int e = a + lane * 4;
+    float wv[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) wv[q] = e + q < b ? __ldg(w + e + q) : 0.0f;
+    if (a < b) race_chunk(R, wv, (wv[0] + wv[1]) + (wv[2] + wv[3]), a, lane, seed, r, stream);
+    return R;
+}
+
+template <int K, bool SHORT>
 __device__ int draw_expj(Group<K>& G, const float* __restrict__ w, int64_t n, uint64_t seed, uint64_t r) {
     const int lane = G.tid & 31;
     const bool vec = ((uintptr_t)w & 15) == 0;
-    if (K == 32) return race_segment(w, 0, n, lane, seed, r, 0, vec).sel;
+    if (K == 32) return SHORT ? race_short(w, 0, (int)n, lane, seed, r, 0).sel : race_segment(w, 0, n, lane, seed, r, 0, vec).sel;
     // CTA width: K / 32 contiguous segments (multiples of 128 entries)
     const int wp = G.tid >> 5;
     const int64_t seg = ((n + K / 32 - 1) / (K / 32) + 127) / 128 * 128;
     const int64_t a = min(n, (int64_t)wp * seg), b = min(n, a + seg);
-    const Race R = race_segment(w, a, b, lane, seed, r, (uint32_t)wp, vec);
+    const Race R = SHORT ? race_short(w, (int)a, (int)b, lane, seed, r, (uint32_t)wp)
+                         : race_segment(w, a, b, lane, seed, r, (uint32_t)wp, vec);
     __shared__ unsigned long long best;
     if (G.tid == 0) best = ~0ull;
     __syncthreads();
@@ -450,9 +469,18 @@ __device__ int draw_expj(Group<K>& G, const float* __restrict__ w, int64_t n, ui
     return bv == ~0ull ? -1 : (int)(bv & 0xFFFFFFFFull);
 }
 
-template <int METHOD, int K>
-__global__ void __launch_bounds__(256, METHOD == SAMP_EXPJ ? 5 : 8) sampler_kernel(const float* __restrict__ w, int64_t n, int64_t reps,
-                                                      uint64_t seed, int32_t* __restrict__ out) {
+// Each form of a sampler is a kernel of its own, with the registers it needs (2^18
+// draws of 200 weights at warp width by DPRS: 174 us, 195 with all in one kernel):
+// one chunk or element per thread (SHORT), few (FEW), any number (LONG).  CTAs
+// per SM: the four-chunk race needs 48 registers, a single chunk 40; at CTA
+// width 32 with a few spills are better there, as the barriers want more warps
+// (2^18 draws of 32 weights: 462 us against 533).
+enum Form { SHORT, FEW, LONG };
+template <int METHOD, int K, Form FORM>
+__global__ void __launch_bounds__(256, METHOD == SAMP_EXPJ && FORM == LONG   ? 5
+                                       : K == 32 && METHOD == SAMP_EXPJ ? 6
+                                       : 8) sampler_kernel(
+    const float* __restrict__ w, int64_t n, int64_t reps, uint64_t seed, int32_t* __restrict__ out) {
     __shared__ float fbuf[64];
     __shared__ int ibuf[8];
     Group<K> G;
@@ -463,33 +491,44 @@ __global__ void __launch_bounds__(256, METHOD == SAMP_EXPJ ? 5 : 8) sampler_kern
     const int gi = (int)(threadIdx.x / K);
     for (int64_t r = (int64_t)blockIdx.x * groups + gi; r < reps; r += (int64_t)gridDim.x * groups) {
         int sel;
-        // (the lines between the three lie where they measured equal)
-        constexpr int64_t kFew = K == 32 ? 256 : 768;
-        if (METHOD == SAMP_EXPJ) sel = draw_expj<K>(G, w, n, seed, (uint64_t)r);
-        else if (n <= K) sel = draw_short<K, METHOD == SAMP_ZPRS>(G, w, (uint32_t)n, seed, (uint64_t)r);
+        if (METHOD == SAMP_EXPJ) sel = draw_expj<K, FORM == SHORT>(G, w, n, seed, (uint64_t)r);
+        else if (FORM == SHORT) sel = draw_short<K, METHOD == SAMP_ZPRS>(G, w, (uint32_t)n, seed, (uint64_t)r);
         else if (METHOD == SAMP_DPRS)
-            sel = n <= kFew ? draw_dprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
-                            : draw_dprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
+            sel = FORM == FEW ? draw_dprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
+                              : draw_dprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
         else
-            sel = n <= kFew ? draw_zprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
-                            : draw_zprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
+            sel = FORM == FEW ? draw_zprs_few<K>(G, w, (uint32_t)n, seed, (uint64_t)r)
+                              : draw_zprs<K>(G, w, (uint32_t)n, seed, (uint64_t)r);
         if (G.tid == 0) out[r] = sel;
     }
 }
 
-template <int METHOD, int K>
-cudaError_t launch_sampler(const float* w, int64_t n, int64_t reps, uint64_t seed, int32_t* out, cudaStream_t st) {
+template <int METHOD, int K, Form FORM>
+cudaError_t launch_form(const float* w, int64_t n, int64_t reps, uint64_t seed, int32_t* out, cudaStream_t st) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sampler_kernel<METHOD, K>, 256, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sampler_kernel<METHOD, K, FORM>, 256, 0);
     if (e != cudaSuccess) return e;
     const int64_t groups = 256 / K;
     int64_t grid = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
     const int64_t need = (reps + groups - 1) / groups;
     if (need < grid) grid = need;
-    sampler_kernel<METHOD, K><<<(unsigned)grid, 256, 0, st>>>(w, n, reps, seed, out);
+    sampler_kernel<METHOD, K, FORM><<<(unsigned)grid, 256, 0, st>>>(w, n, reps, seed, out);
     return cudaGetLastError();
+}
+
+template <int METHOD, int K>
+cudaError_t launch_sampler(const float* w, int64_t n, int64_t reps, uint64_t seed, int32_t* out, cudaStream_t st) {
+    // (the lines between few and many lie where the two measured equal)
+    constexpr int64_t kShort = METHOD != SAMP_EXPJ ? K : K == 32 ? 128 : 1024;  // the race: one chunk per warp
+    constexpr int64_t kFew = METHOD == SAMP_EXPJ ? 0 : K == 32 ? 256 : 768;
+    if (n <= kShort) return launch_form<METHOD, K, SHORT>(w, n, reps, seed, out, st);
+    // (ZPRS at CTA width: five iterations cost less than two groups of four, for
+    // 1,025 weights 499 us against 540, up to about here)
+    const bool five = METHOD == SAMP_ZPRS && K == 256 && n > 4 * K && n <= 4 * K + K / 2;
+    if (METHOD != SAMP_EXPJ && (n <= kFew || five)) return launch_form<METHOD, K, METHOD == SAMP_EXPJ ? LONG : FEW>(w, n, reps, seed, out, st);
+    return launch_form<METHOD, K, LONG>(w, n, reps, seed, out, st);
 }
 
 }  // namespace

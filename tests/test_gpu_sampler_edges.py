@@ -118,3 +118,22 @@ def test_reservoir_law(width, n):
     p = w.double().cpu().numpy()
     _, pv = chi2_tv(np.bincount(got.cpu().numpy(), minlength=n), p / p.sum(), draws)
     assert pv > 1e-6, (n, pv)
+
+
+@pytest.mark.parametrize("width", [32, 256])
+@pytest.mark.parametrize("n", [1, 2, 5, 64, 127, 128])
+def test_short_reservoir_draws_as_the_general_one(width, n):
+    """Zeros behind the weights are never drawn, but lead past the one-chunk kernel."""
+    need_gpu()
+    built()
+    from paper_2404_08364_gb300 import sample
+    w = _weights(n, n % 2 == 1)
+    padded = torch.cat([w, torch.zeros((128 if width == 32 else 1024) + 1 - n, device=w.device)])
+    a, _ = sample("expj", w, 4099, seed=SEED, width=width)
+    b, _ = sample("expj", padded, 4099, seed=SEED, width=width)
+    assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025])
+def test_reservoir_law_where_segments_grow(n):
+    test_reservoir_law(256, n)
