@@ -2,8 +2,9 @@
 // re-designed for sm_103a without block-wide barriers).
 //
 // Scheduling (Section 5's sampler-centric model and two-level task pools):
-//   * Every warp is an independent sampler with a few walk slots of its own
-//     in shared memory (its share of the CTA's local task pool P_L).  It
+//   * Every warp is an independent sampler with a walk slot of its own (more
+//     if the caller asks) in shared memory: its share of the CTA's local task
+//     pool P_L.  It
 //     claims queries from one global atomic cursor over the callers' request
 //     arrays (the global task pool P_G: nothing extra in global memory) and
 //     runs one step at a time on whichever of its walks is ready.
@@ -32,7 +33,8 @@
 // scanned again (a row of one pair is picked from at once).  Measured on the
 // R-MAT-20 node2vec batch of 2^15 walks: 69.8 ms with per-128-entry sums, rows
 // above 8,184 entries as hub tasks and 136 KB of code (the warps waited for
-// instructions 55 % of their time), 12.7 ms on this engine.
+// instructions 55 % of their time), 10.1 ms on this engine (4.2 ms at copy
+// bandwidth; it is bound by instruction issue in the membership test).
 //
 // First-order rules (weighted, MetaPath, PPR) need a row's weights (and
 // labels) and the one picked column, so only those are read: 4 (5) bytes per
@@ -43,7 +45,9 @@
 // 37.9 ms with columns and weights through a TMA ring on 16 warps per SM,
 // 22.6 ms with the weights alone through the ring on 32, 21.5 ms by direct
 // loads (180 -> 75 instructions per 512 entries: no barrier waits, refills and
-// shared round trip), 19.5 ms with the per-step code cut down.
+// shared round trip), 19.5 ms with the per-step code cut down, 14.1 ms with all
+// weights in registers, one walk per warp and records through shared memory.
+// 12.9 ms is what the weights take at copy bandwidth.
 #pragma once
 
 #include "fw_device.cuh"
