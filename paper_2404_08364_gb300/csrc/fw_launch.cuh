@@ -9,11 +9,16 @@
 namespace fw {
 namespace {
 
+constexpr int kSmemLimit = 227 * 1024;  // dynamic shared memory a CTA may have
+
 // Grid and shared memory of one engine launch: every SM filled as far as the
 // kernel's registers and shared memory allow (at most tu.ctas_per_sm CTAs each).
 template <typename K>
 cudaError_t engine_grid(K kern, int threads, size_t smem, const Tuning& tu, int* sms, int* per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // always the same limit: it belongs to the function, and another thread may be
+    // about to launch the same kernel with more than this call needs
+    if (smem > (size_t)kSmemLimit) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     int dev = 0;
     cudaGetDevice(&dev);
