@@ -998,6 +998,10 @@ __device__ __noinline__ int claim_query(const GraphDev& g, const ReqDev* __restr
             atomicAdd(&L.counters[C_BAD_INPUT], 1ull);
             st = ST_FINISH;  // written out as an empty path
         } else {
+            // the walk that ended in this slot may have left its last row's
+            // copies open (commit asks for them before it knows whether the
+            // walk goes on); two copies into the same words have no order
+            cp_async_wait_all();
             fetch_row(g, sl, start);
             Rq.paths[qi * ((long long)Rq.max_len + 1)] = start;
             sl.k = 1;
