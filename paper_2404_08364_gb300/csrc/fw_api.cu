@@ -79,7 +79,11 @@ struct CheckOut {
     unsigned long long descents;      // entries i with col[i] >= col[i + 1]
     unsigned long long at_row_starts; // those whose i + 1 is the first entry of a row
 };
-static_assert(sizeof(CheckOut) <= sizeof(Scratch), "the checks' results go to the graph's scratch");
+// What precedes the arrays in a graph's allocation.
+struct Head {
+    Scratch scratch;
+    CheckOut check;
+};
 
 // Row offsets: one thread per row, so every offset is read once.  Whether the
 // rows ascend is decided over the whole column array: it does exactly if every
@@ -236,7 +240,7 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
     // One allocation holds everything.  Three for 1.06 GB (R-MAT-22's offsets,
     // columns and one array of weights) took 313 us and their release 717 us,
     // one 150 and 515; load, a walk of 0.6 ms and release: 3.06 -> 2.66 ms.
-    const size_t head = (sizeof(Scratch) + 255) & ~(size_t)255;
+    const size_t head = (sizeof(Head) + 255) & ~(size_t)255;
     size_t bytes = head;
     if (!borrow)
         bytes += held_bytes(row_ptr, n + 1, 8) + held_bytes(col, m, 4) + held_bytes(w_f32, m, 4) + held_bytes(w_u32, m, 4) +
@@ -247,7 +251,8 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
         release(G);
         return fail(e == cudaErrorMemoryAllocation ? FW_ENOMEM : FW_ECUDA, "fw_load_csr: allocation: %s", cudaGetErrorString(e));
     }
-    G->scratch = reinterpret_cast<Scratch*>(G->mem);
+    Head* hd = reinterpret_cast<Head*>(G->mem);
+    G->scratch = &hd->scratch;
     if (borrow) {
         G->g.row_ptr = row_ptr;
         G->g.col = col;
@@ -266,7 +271,7 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
             return rc;
         }
     }
-    if (cudaMemset(G->scratch, 0, sizeof(Scratch)) != cudaSuccess) {
+    if (cudaMemset(hd, 0, sizeof(Head)) != cudaSuccess) {
         release(G);
         return fail(FW_ENOMEM, "fw_load_csr: scratch allocation");
     }
@@ -276,8 +281,11 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
     }
 
     // ---- checks (and the max degree / max integer weight) on the device ----
-    // (their results lie in the scratch, which is cleared again behind them)
-    CheckOut* dco = reinterpret_cast<CheckOut*>(G->scratch);
+    // Their results have a place of their own behind the scratch, and reading
+    // them back is the last thing queued here: it waits for the clear above,
+    // which no stream of a later walk does (a clear of device memory returns
+    // before it has run).
+    CheckOut* dco = &hd->check;
     CheckOut co = {};
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, G->device);
@@ -287,7 +295,6 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
         check_entries_kernel<<<(unsigned)(entry_blocks < sms * 8 ? entry_blocks : sms * 8), 256>>>(
             G->g.col, G->g.w_f32, G->g.w_u32, n, m, dco);
     e = cudaMemcpy(&co, dco, sizeof co, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemset(G->scratch, 0, sizeof(Scratch));
     if (e != cudaSuccess) {
         release(G);
         return fail(FW_ECUDA, "fw_load_csr: checks: %s", cudaGetErrorString(e));
