@@ -916,7 +916,9 @@ __device__ __noinline__ int hub_claim(CtaHead& H0, int lane) {
         }
         __threadfence_block();
     }
-    return __shfl_sync(FULL, got, 0);
+    got = __shfl_sync(FULL, got, 0);
+    __syncwarp();  // the other lanes read the task behind lane 0's fence (a shuffle orders no memory)
+    return got;
 }
 
 // The step's 64-bit draw (exact mode).
@@ -1108,6 +1110,7 @@ __device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restric
         // another warp may flip a hub-parked slot at any time: let lane 0
         // read it once for the whole warp
         int st = __shfl_sync(FULL, *(volatile int*)&sl.state, 0);
+        __syncwarp();
         if (st == ST_EMPTY && !wh.exhausted) {
             st = claim_query<N2V, SERVE>(g, reqs, L, sv, sl, lane);
             if (st < 0) {
@@ -1282,10 +1285,13 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
             if (seg >= 0 && lane == 0) {
                 // fold the segment into its hub task; the warp that completes
                 // the last segment finishes the step
+                // (the count is read first: once this segment is added, the
+                // task may be finished, freed and another one's)
                 HubTask& H = head.hub[seg >> 8];
+                const int nseg = hub_nseg(*(volatile unsigned*)&H.ctl);
                 if (best != ~0ull) atomicMin(&H.best, best);
                 __threadfence_block();
-                fin = atomicAdd(&H.done_seg, 1) == hub_nseg(*(volatile unsigned*)&H.ctl) - 1;
+                fin = atomicAdd(&H.done_seg, 1) == nseg - 1;
                 __threadfence_block();
                 best = *(volatile unsigned long long*)&H.best;
             }
@@ -1329,7 +1335,9 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
                         last = atomicAdd(&H.done_seg, 1) == nseg - 1;
                         __threadfence_block();
                     }
-                    if (!__shfl_sync(FULL, last, 0)) {
+                    last = __shfl_sync(FULL, last, 0);
+                    __syncwarp();  // every lane reads the other warps' totals behind lane 0's fence
+                    if (!last) {
                         fin = false;
                         break;
                     }
