@@ -1037,6 +1037,7 @@ __device__ __noinline__ void retire_walk(const ServeDev& sv, Slot& sl, unsigned 
     int32_t* row = Rq.paths + sl.q * width;
 #pragma unroll 1
     for (long long e = k + lane; e < width; e += 32) row[e] = -1;
+    if (SERVE) __syncwarp();  // lane 0's fence below is to cover every lane's padding
     if (lane == 0) {
         Rq.path_len[sl.q] = k;
         cnt[N_WALKS] += 1;
