@@ -370,6 +370,9 @@ extern "C" int fw_server_create(fw_graph* graph, int32_t mode, uint64_t mem_budg
         chk(cudaMemset(S->stop, 0, sizeof(int)));
         chk(cudaMemset(S->scratch, 0, sizeof(Scratch)));
         chk(cudaMemset(S->done, 0, sizeof(unsigned long long) * (size_t)S->maxr));
+        // (the clears return before they have run, and the server's own
+        // streams do not wait for the one they are queued on)
+        chk(cudaStreamSynchronize(0));
     }
     if (e != cudaSuccess) {
         fw_server_destroy(S);
