@@ -379,7 +379,8 @@ int fw_autotune_clear_cache(void);
 int fw_set_tuning(fw_graph* g, const fw_tuning* t);
 int fw_get_tuning(const fw_graph* g, fw_tuning* out);
 
-/* Synchronise the graph's last stream and copy the counters to *out. */
+/* Wait for the graph's last launch, replay and counter reset and copy the
+ * counters to *out. */
 int fw_stats(fw_graph* g, fw_stats_t* out);
 int fw_stats_reset(fw_graph* g, void* stream);
 

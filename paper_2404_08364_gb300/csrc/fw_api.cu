@@ -60,8 +60,8 @@ struct fw_graph {
     uint32_t max_w_u32;
     Scratch* scratch;          // device: cursor + counters
     Tuning tuning;
-    cudaStream_t last_stream;
-    cudaEvent_t ev0, ev1;
+    cudaEvent_t ev0, ev1;      // around the last direct launch
+    cudaEvent_t mark;          // behind the last replay or reset of the counters
     bool timed;
     std::mutex mu;
 };
@@ -207,6 +207,7 @@ void release(fw_graph* G) {
     if (G->mem) cudaFree(G->mem);
     if (G->ev0) cudaEventDestroy(G->ev0);
     if (G->ev1) cudaEventDestroy(G->ev1);
+    if (G->mark) cudaEventDestroy(G->mark);
     cudaSetDevice(cur);
     delete G;
 }
@@ -275,7 +276,8 @@ extern "C" int fw_load_csr(fw_graph** out, int64_t n, int64_t m, const int64_t* 
         release(G);
         return fail(FW_ENOMEM, "fw_load_csr: scratch allocation");
     }
-    if (cudaEventCreate(&G->ev0) != cudaSuccess || cudaEventCreate(&G->ev1) != cudaSuccess) {
+    if (cudaEventCreate(&G->ev0) != cudaSuccess || cudaEventCreate(&G->ev1) != cudaSuccess ||
+        cudaEventCreateWithFlags(&G->mark, cudaEventDisableTiming) != cudaSuccess) {
         release(G);
         return fail(FW_ECUDA, "fw_load_csr: event creation");
     }
@@ -415,7 +417,6 @@ int launch(fw_graph* G, int mode, const ReqTable& tab, int n_req, int64_t total,
     if (e != cudaSuccess) return fail(FW_ECUDA, "walk launch: %s", cudaGetErrorString(e));
     if (timed) FW_CUDA_TRY(cudaEventRecord(G->ev1, st));
     G->timed = timed;
-    G->last_stream = st;
     return FW_OK;
 }
 
@@ -439,6 +440,13 @@ int make_request(const fw_graph* g, const fw_request& q, ReqDev* out) {
 Scratch* graph_scratch(const fw_graph* g) { return g->scratch; }
 
 std::mutex& graph_mutex(fw_graph* g) { return g->mu; }
+
+int graph_mark(fw_graph* g, cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(stream, &cap);
+    if (cap == cudaStreamCaptureStatusNone) FW_CUDA_TRY(cudaEventRecord(g->mark, stream));
+    return FW_OK;
+}
 
 }  // namespace fw
 
@@ -587,7 +595,10 @@ extern "C" int fw_sync(void* stream) {
 extern "C" int fw_stats(fw_graph* G, fw_stats_t* out) {
     if (!G || !out) return fail(FW_EINVAL, "fw_stats: NULL argument");
     std::lock_guard<std::mutex> lock(G->mu);
-    cudaError_t e = cudaStreamSynchronize(G->last_stream);
+    // (events, not the streams: a stream that a launch was captured or tuned on
+    // is gone by now)
+    cudaError_t e = cudaEventSynchronize(G->ev1);
+    if (e == cudaSuccess) e = cudaEventSynchronize(G->mark);
     if (e != cudaSuccess) return fail(FW_ECUDA, "fw_stats: %s", cudaGetErrorString(e));
     Scratch s;
     e = cudaMemcpy(&s, G->scratch, sizeof s, cudaMemcpyDeviceToHost);
@@ -620,8 +631,7 @@ extern "C" int fw_stats_reset(fw_graph* G, void* stream) {
     if (!G) return fail(FW_EINVAL, "fw_stats_reset: NULL graph");
     std::lock_guard<std::mutex> lock(G->mu);
     FW_CUDA_TRY(cudaMemsetAsync(G->scratch, 0, sizeof(Scratch), (cudaStream_t)stream));
-    G->last_stream = (cudaStream_t)stream;
-    return FW_OK;
+    return graph_mark(G, (cudaStream_t)stream);
 }
 
 // -------------------------------------------------------- Philox cross-check
@@ -744,6 +754,5 @@ extern "C" int fw_walk_noalloc(fw_graph* G, const fw_request* reqs, int32_t n_re
     if (e != cudaSuccess) return fail(FW_ECUDA, "fw_walk_noalloc: launch: %s", cudaGetErrorString(e));
     if (timed) FW_CUDA_TRY(cudaEventRecord(G->ev1, st));
     G->timed = timed;
-    G->last_stream = st;
     return FW_OK;
 }

@@ -198,5 +198,6 @@ int graph_device_view(const fw_graph* g, GraphDev* out, int* device, Tuning* tun
 int make_request(const fw_graph* g, const fw_request& q, ReqDev* out);  // parameters only
 Scratch* graph_scratch(const fw_graph* g);                            // the graph's cursor and counters
 std::mutex& graph_mutex(fw_graph* g);                                 // serialises launches on the graph
+int graph_mark(fw_graph* g, cudaStream_t stream);                     // fw_stats waits for what is queued here (under the mutex)
 
 }  // namespace fw

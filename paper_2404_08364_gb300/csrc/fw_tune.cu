@@ -58,6 +58,7 @@ std::string cache_key(const fw_graph* g, const fw_request* reqs, int n_req) {
 }  // namespace
 
 struct fw_exec {
+    fw_graph* owner = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -69,6 +70,7 @@ extern "C" int fw_capture_multi(fw_graph* g, const fw_request* reqs, int32_t n_r
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess)
         return fail_t(FW_ECUDA, "fw_capture_multi: stream creation failed");
     fw_exec* X = new fw_exec();
+    X->owner = g;
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed);
     int rc = e == cudaSuccess ? fw_walk_multi(g, reqs, n_req, st) : FW_ECUDA;
     cudaError_t e2 = cudaStreamEndCapture(st, &X->graph);
@@ -87,7 +89,8 @@ extern "C" int fw_exec_launch(fw_exec* X, void* stream) {
     if (!X || !X->exec) return fail_t(FW_EINVAL, "fw_exec_launch: NULL exec");
     cudaError_t e = cudaGraphLaunch(X->exec, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail_t(FW_ECUDA, "fw_exec_launch: %s", cudaGetErrorString(e));
-    return FW_OK;
+    std::lock_guard<std::mutex> lk(graph_mutex(X->owner));
+    return graph_mark(X->owner, (cudaStream_t)stream);
 }
 
 extern "C" void fw_exec_destroy(fw_exec* X) {
