@@ -29,10 +29,11 @@ int fail_b(int status, const char* fmt, ...) {
     return set_error(status, buf);
 }
 
-// dst counters += src counters (the cursor is not a counter).
+// dst counters += src counters (the cursor is not a counter).  Atomically: a walk
+// on one of the caller's streams may still be adding to dst.
 __global__ void add_counters_kernel(Scratch* dst, const Scratch* a, const Scratch* b) {
     const int i = threadIdx.x;
-    if (i < C_NUM) dst->counters[i] += a->counters[i] + b->counters[i];
+    if (i < C_NUM) atomicAdd(&dst->counters[i], a->counters[i] + b->counters[i]);
 }
 
 // Bytes one query needs in one pool: its path (L + 1 vertices), its start
