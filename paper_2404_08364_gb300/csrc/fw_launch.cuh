@@ -71,7 +71,10 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
         // (a warp advances its walks one after another), spread evenly over
         // the CTAs.  Hub rows begin at one segment (fast mode) or where the
         // pieces are still worth a hand-off (exact mode); where the graph has
-        // such rows, one large CTA per SM keeps warps at hand for them.
+        // such rows, one large CTA per SM keeps warps at hand for them, as long
+        // as its 24 warps hold all walks: a first-order launch of 25 to 32 walks
+        // per SM would run the rest as a second round (4,800 weighted walks of
+        // 80 on R-MAT-22, fast 1,416 us with the large CTAs, 1,152 without).
         // Measured (us): 1,000 exact walks of 80 on a 1,000-vertex graph 617
         // (four walks per warp) -> 222; 32 node2vec walks of 40 on R-MAT-22,
         // fast 868 -> 777, exact 1,095 -> 712 (helpers); 129 PPR walks on
@@ -82,9 +85,13 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
             L.seg_q = 512;
         }
         if (!own && g.d_max > d_t) {
-            threads = 768;
-            e = engine_grid(kern, threads, cta_smem<EXACT, N2V>(threads / 32, use), tu, &sms, &per_sm);
+            int wide = 0;
+            e = engine_grid(kern, 768, cta_smem<EXACT, N2V>(24, use), tu, &sms, &wide);
             if (e != cudaSuccess) return e;
+            if (total <= (int64_t)sms * wide * 24) {
+                threads = 768;
+                per_sm = wide;
+            }
         }
         grid = min((int64_t)sms * per_sm, total);
         L.claimers = (int)((total + grid - 1) / grid);
