@@ -107,19 +107,20 @@ typedef struct {
 /*
  * Engine tuning (Section 5.1's |P_L| and d_t and the launch shape).
  *   block_threads   threads per CTA: 128, 256 or 512 (anything else: the
- *                   default, 512, which leaves the shape to the engine while
- *                   ctas_per_sm is 0 too).
+ *                   default, 256, or 512 if ctas_per_sm is set.  At 256, with
+ *                   ctas_per_sm 0, launches of few walks take larger CTAs).
  *   slots           walks resident per CTA: the local task pool P_L, at most
- *                   8 per warp (default, nominally, 4 per warp; while it is
- *                   not set the engine runs one).
+ *                   8 per warp (default: one per warp; counted per 512
+ *                   threads while block_threads is not set).
  *   d_warp          degree threshold d_t: rows with d <= d_warp are sampled
  *                   by one warp, larger rows by the whole CTA (default 65536;
- *                   while it is not set, a batch launch also shares rows above
+ *                   at the default, a batch launch also shares rows above
  *                   16384 entries, in small exact launches above 4096, once a
  *                   warp of the CTA has no walk left, and in fast mode it
  *                   shares no others).
  *   ctas_per_sm     persistent CTAs per SM (0 = as many as fit).
- * Zero fields mean "default".  No field changes a walk's result: exact mode is
+ * Zero fields mean "default".  fw_get_tuning returns the values in force, and
+ * setting them again changes nothing.  No field changes a walk's result: exact mode is
  * bit-identical to the CPU oracle under every tuning, and fast mode draws each
  * row with the same segment streams whichever sampler takes it.
  */
@@ -369,7 +370,8 @@ void fw_exec_destroy(fw_exec* x);
  * walk steps per second, sets it on g and returns it in *best (and its rate in
  * *best_steps_per_s when not NULL).  The choice is cached by (GPU name,
  * algorithms and mode of the sample, log2 mean and max degree of g); a cache
- * hit returns at once with rate 0.  1 <= n_req <= 16.
+ * hit returns at once with rate 0.  1 <= n_req <= 16.  On an error g keeps the
+ * tuning it had.
  */
 int fw_autotune(fw_graph* g, const fw_request* reqs, int32_t n_req, int32_t reps, fw_tuning* best,
                 double* best_steps_per_s);

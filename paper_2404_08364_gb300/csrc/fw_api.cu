@@ -337,7 +337,7 @@ extern "C" int fw_graph_info(const fw_graph* g, int64_t* n, int64_t* m, int64_t*
 extern "C" int fw_set_tuning(fw_graph* g, const fw_tuning* t) {
     if (!g) return fail(FW_EINVAL, "fw_set_tuning: NULL graph");
     Tuning tu = default_tuning();
-    if (t) tu = Tuning{t->block_threads, t->slots, t->d_warp, t->ctas_per_sm, true, true, true};
+    if (t) tu = Tuning{t->block_threads, t->slots, t->d_warp, t->ctas_per_sm};
     g->tuning = sanitize_tuning(tu);
     return FW_OK;
 }

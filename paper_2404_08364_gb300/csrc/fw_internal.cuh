@@ -149,14 +149,16 @@ struct ServeDev {
 
 constexpr unsigned long long kTakenBase = 1ull << 62;
 
+// A field at its default leaves the choice to the launch (fw_launch.cuh), whether
+// the caller set it to that or not at all: so reading a tuning and setting it
+// again changes nothing.
 struct Tuning {
     int block_threads;
     int slots;
     int d_warp;
     int ctas_per_sm;
-    bool own_slots;  // slots was set by the caller (else one walk per warp)
-    bool own_d;      // d_warp was set by the caller
-    bool own_shape;  // block_threads was set by the caller (else each engine may take the CTA size that suits it)
+    bool own_shape() const { return block_threads != 256 || ctas_per_sm > 0; }
+    bool own_d() const { return d_warp != 65536; }
 };
 
 // Launch the persistent walk engine over `n_req` requests (device array

@@ -36,7 +36,7 @@ cudaError_t engine_grid(K kern, int threads, size_t smem, const Tuning& tu, int*
 // node2vec R-MAT-25 187.1 -> 182.4, R-MAT-20 35.8 -> 33.1, exact 12.9 -> 10.4,
 // weighted R-MAT-22 15.8 -> 15.0, MetaPath + PPR 7.9 -> 7.3.
 inline int walks_per_warp(const Tuning& tu) {
-    return tu.own_slots ? max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32))) : 1;
+    return max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
 }
 
 template <bool EXACT, bool N2V, bool LAB>
@@ -48,8 +48,7 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
     // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
     // (R-MAT-25 node2vec: 240 -> 202 ms), and a hub row's last segments hold
     // back 8 warps instead of 16 (PPR from the R-MAT-22 hub: 5.7 -> 4.8 ms).
-    const bool own = tu.own_shape || tu.ctas_per_sm > 0;
-    int threads = own ? tu.block_threads : 256, use = sw;
+    int threads = tu.block_threads, use = sw;
     int sms = 0, per_sm = 0;
     cudaError_t e = engine_grid(kern, threads, cta_smem<EXACT, N2V>(threads / 32, sw), tu, &sms, &per_sm);
     if (e != cudaSuccess) return e;
@@ -57,7 +56,7 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
     int64_t grid = (int64_t)sms * per_sm;
     Launch L = {reqs.ext, n_req, (long long)total, cursor, counters, tu.d_warp, threads / 32, kSegQuads, 4096u};
     int d_t = tu.d_warp;
-    if (!tu.own_d) {
+    if (!tu.own_d()) {
         // Sharing a row costs throughput (hand-offs, fresh N(prev) cursors,
         // waiting owners) and gains latency: unless the caller set d_t, rows
         // from one segment on are shared while the CTA has a warp without walks
@@ -80,11 +79,11 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
         // fast 868 -> 777, exact 1,095 -> 712 (helpers); 129 PPR walks on
         // R-MAT-22 222 -> 201.
         use = 1;
-        if (!tu.own_d && EXACT) {
+        if (!tu.own_d() && EXACT) {
             d_t = 4096;
             L.seg_q = 512;
         }
-        if (!own && g.d_max > d_t) {
+        if (!tu.own_shape() && g.d_max > d_t) {
             int wide = 0;
             e = engine_grid(kern, 768, cta_smem<EXACT, N2V>(24, use), tu, &sms, &wide);
             if (e != cudaSuccess) return e;
@@ -126,8 +125,7 @@ cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, 
     // Filling every SM would hold those back for as long as the server runs,
     // and through the hardware queues streams share, the server's own copies
     // queued behind them.
-    const int warps = 24;
-    const int sw = walks_per_warp(tu);
+    const int warps = 24, sw = 1;
     const size_t smem = cta_smem<EXACT, true>(warps, sw);
     int sms = 0, per_sm = 0;
     cudaError_t e = engine_grid(kern, warps * 32, smem, tu, &sms, &per_sm);

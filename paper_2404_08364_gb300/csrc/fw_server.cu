@@ -326,14 +326,11 @@ extern "C" int fw_server_create(fw_graph* graph, int32_t mode, uint64_t mem_budg
     fw_server* S = new fw_server();
     S->graph = graph;
     graph_device_view(graph, &S->g, &S->device, &S->tuning);
-    // The resident engine runs one CTA per SM, one walk per warp, whatever
-    // the graph's batch tuning (that tuning's d_t is kept; no tuning changes a
-    // result), and leaves eight SMs free for other streams' kernels: 768
-    // threads in fast mode (a burst of 24 mixed requests on R-MAT-22, server
-    // start to last result: 33.4 ms with the earlier engine's 512, 16.7 ms
-    // now), 512 in exact mode.
-    S->tuning.block_threads = 512;
-    S->tuning.own_slots = false;
+    // The resident engine runs one 768-thread CTA per SM, one walk per warp,
+    // whatever the graph's batch tuning (that tuning's d_t is kept; no tuning
+    // changes a result), and leaves eight SMs free for other streams' kernels (a
+    // burst of 24 mixed requests on R-MAT-22, server start to last result: 33.4
+    // ms with the earlier engine's 512 threads, 16.7 ms now).
     S->tuning.ctas_per_sm = 0;
     S->mode = mode;
     S->maxr = max_requests;

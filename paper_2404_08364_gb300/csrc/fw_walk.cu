@@ -3,23 +3,20 @@
 
 namespace fw {
 
-Tuning default_tuning() { return Tuning{512, 64, 65536, 0, false, false, false}; }
+Tuning default_tuning() { return Tuning{256, 8, 65536, 0}; }
 
 Tuning sanitize_tuning(Tuning t) {
     const Tuning d = default_tuning();
+    // (a caller who limits the CTAs per SM gets large ones; slots without a CTA
+    // size are counted per 512 threads, whatever size the engine takes)
     if (t.block_threads != 128 && t.block_threads != 256 && t.block_threads != 512) {
-        t.block_threads = d.block_threads;
-        t.own_shape = false;
+        t.block_threads = t.ctas_per_sm > 0 ? 512 : d.block_threads;
+        if (t.slots > 0) t.slots = (t.slots > 16 ? t.slots / 16 : 1) * (t.block_threads / 32);
     }
-    if (t.slots <= 0) {
-        t.slots = 4 * (t.block_threads / 32);  // (nominal)
-        t.own_slots = false;
-    }
-    if (t.slots > (t.block_threads / 32) * kSlotsPerWarp) t.slots = (t.block_threads / 32) * kSlotsPerWarp;
-    if (t.d_warp <= 0) {
-        t.d_warp = d.d_warp;
-        t.own_d = false;
-    }
+    const int warps = t.block_threads / 32;
+    if (t.slots <= 0) t.slots = warps;
+    if (t.slots > warps * kSlotsPerWarp) t.slots = warps * kSlotsPerWarp;
+    if (t.d_warp <= 0) t.d_warp = d.d_warp;
     if (t.d_warp < 128) t.d_warp = 128;
     if (t.d_warp > (1 << 30)) t.d_warp = 1 << 30;
     if (t.ctas_per_sm < 0) t.ctas_per_sm = 0;
