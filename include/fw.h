@@ -365,8 +365,8 @@ void fw_exec_destroy(fw_exec* x);
 /*
  * Engine autotuner (Section 5.1's |P_L| and d_t, and the CTA size): runs
  * fw_walk_multi(reqs) — a representative sample of the workload, device
- * buffers — over a grid of tunings (128/256/512 threads, d_t 2^11 .. 2^20,
- * 1..4 walk slots per warp), `reps` timed launches each, keeps the fastest in
+ * buffers — with the default tuning and over a grid of others (128/256/512
+ * threads, d_t 2^11 .. 2^20, 1..4 walk slots per warp), `reps` timed launches each, keeps the fastest in
  * walk steps per second, sets it on g and returns it in *best (and its rate in
  * *best_steps_per_s when not NULL).  The choice is cached by (GPU name,
  * algorithms and mode of the sample, log2 mean and max degree of g); a cache

@@ -129,31 +129,33 @@ extern "C" int fw_autotune(fw_graph* g, const fw_request* reqs, int32_t n_req, i
     double best_rate = -1.0;
     fw_tuning best_t = saved;
     int rc = FW_OK;
+    // the default launch first: tuning never ends with less than it
+    std::vector<fw_tuning> grid(1, fw_tuning{0, 0, 0, 0});
     for (int nt : threads)
         for (int dt : dts)
-            for (int spw : slots_per_warp) {
-                fw_tuning t = {nt, spw * (nt / 32), dt, 0};
-                fw_set_tuning(g, &t);
-                fw_stats_reset(g, st);
-                rc = fw_walk_multi(g, reqs, n_req, st);  // warm-up
-                if (rc != FW_OK) break;
-                fw_stats_reset(g, st);
-                cudaEventRecord(e0, st);
-                for (int r = 0; r < reps && rc == FW_OK; ++r) rc = fw_walk_multi(g, reqs, n_req, st);
-                cudaEventRecord(e1, st);
-                if (rc != FW_OK) break;
-                fw_stats_t s;
-                rc = fw_stats(g, &s);
-                if (rc != FW_OK) break;
-                cudaEventSynchronize(e1);
-                float ms = 0.0f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                const double rate = ms > 0 ? (double)s.steps / (ms * 1e-3) : 0.0;
-                if (rate > best_rate) {
-                    best_rate = rate;
-                    fw_get_tuning(g, &best_t);
-                }
-            }
+            for (int spw : slots_per_warp) grid.push_back(fw_tuning{nt, spw * (nt / 32), dt, 0});
+    for (const fw_tuning& t : grid) {
+        fw_set_tuning(g, &t);
+        fw_stats_reset(g, st);
+        rc = fw_walk_multi(g, reqs, n_req, st);  // warm-up
+        if (rc != FW_OK) break;
+        fw_stats_reset(g, st);
+        cudaEventRecord(e0, st);
+        for (int r = 0; r < reps && rc == FW_OK; ++r) rc = fw_walk_multi(g, reqs, n_req, st);
+        cudaEventRecord(e1, st);
+        if (rc != FW_OK) break;
+        fw_stats_t s;
+        rc = fw_stats(g, &s);
+        if (rc != FW_OK) break;
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        const double rate = ms > 0 ? (double)s.steps / (ms * 1e-3) : 0.0;
+        if (rate > best_rate) {
+            best_rate = rate;
+            fw_get_tuning(g, &best_t);
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaStreamDestroy(st);
