@@ -16,7 +16,11 @@ using namespace fw;
 
 static thread_local char g_last_error[512] = "";
 
+// (Every failure of the library ends here.  A CUDA call's error is reported by
+// the status; left behind as the runtime's last error, the next launch of this
+// thread would find it and take it for its own.)
 static int fail(int status, const char* fmt, ...) {
+    if (status == FW_ECUDA || status == FW_ENOMEM) cudaGetLastError();
     va_list ap;
     va_start(ap, fmt);
     vsnprintf(g_last_error, sizeof g_last_error, fmt, ap);
