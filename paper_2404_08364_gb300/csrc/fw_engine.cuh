@@ -1179,12 +1179,15 @@ __device__ __noinline__ int pick_walk(const GraphDev& g, const ReqDev* __restric
     return PICK_AGAIN;
 }
 
-// N2V, LAB: the launch may hold node2vec / MetaPath requests; with N2V, PPR
-// requests need LAB too (a build without them is smaller: see the instruction
-// cache above).
+// N2V, LAB, PPR: the launch may hold node2vec / MetaPath / PPR requests (a build
+// without them is smaller: see the instruction cache above).  Only node2vec
+// launches have a build without PPR.  One with PPR and without labels is worth
+// its place: the label rule sits in every pair's load, and a small node2vec + PPR
+// launch is a chain of those (8 weighted, 32 node2vec and 129 PPR walks on
+// R-MAT-20: 611 us on the build with labels, 577 on this one).
 // SERVE: the served form's build (queries claimed from the request ring,
 // completion stamps, idle polling); the batch build compiles all of that out.
-template <bool EXACT, bool N2V, bool LAB, bool SERVE>
+template <bool EXACT, bool N2V, bool LAB, bool PPR, bool SERVE>
 // Registers: 64 a thread for first-order launches (32 warps per SM), 80 for
 // node2vec (24 warps; 128 registers and 16 warps measured 241 ms against 202
 // on the R-MAT-25 batch of 2^18 walks, 64 registers with spills 248).
@@ -1378,7 +1381,7 @@ __global__ void __maxnreg__(N2V ? 80 : 64)
                 *(volatile int*)&sl.state = ST_FINISH;  // nothing selectable (or a dead end): the walk stops here
             } else {
                 count_step(wh.cnt, (int)(sl.row[1] - sl.row[0]), sl.rq.algo, seg >= 0);
-                commit<LAB || !N2V>(g, sl, sel, seg >= 0);
+                commit<PPR>(g, sl, sel, seg >= 0);
             }
             if (seg >= 0) {
                 __threadfence_block();

@@ -39,10 +39,10 @@ inline int walks_per_warp(const Tuning& tu) {
     return max(1, min(kSlotsPerWarp, tu.slots / (tu.block_threads / 32)));
 }
 
-template <bool EXACT, bool N2V, bool LAB>
+template <bool EXACT, bool N2V, bool LAB, bool PPR>
 cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                       unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
-    auto kern = walk_kernel<EXACT, N2V, LAB, false>;
+    auto kern = walk_kernel<EXACT, N2V, LAB, PPR, false>;
     const int sw = walks_per_warp(tu);
     // CTAs of 256 threads unless the caller chose: at 80 registers three of
     // them fill an SM with 24 warps where 512-thread CTAs leave it at 16
@@ -110,16 +110,15 @@ template <bool EXACT>
 cudaError_t launch_mode(const GraphDev& g, const ReqTable& reqs, int n_req, int64_t total, unsigned long long* cursor,
                         unsigned long long* counters, const Tuning& tu, cudaStream_t stream) {
     const bool n2v = reqs.algos >> FW_NODE2VEC & 1u;
-    const bool lab = reqs.algos >> FW_METAPATH & 1u || (n2v && reqs.algos >> FW_PPR & 1u);
-    return n2v ? (lab ? launch_as<EXACT, true, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
-                      : launch_as<EXACT, true, false>(g, reqs, n_req, total, cursor, counters, tu, stream))
-               : (lab ? launch_as<EXACT, false, true>(g, reqs, n_req, total, cursor, counters, tu, stream)
-                      : launch_as<EXACT, false, false>(g, reqs, n_req, total, cursor, counters, tu, stream));
+    const bool lab = reqs.algos >> FW_METAPATH & 1u, ppr = reqs.algos >> FW_PPR & 1u;
+    const auto as = n2v ? (lab ? launch_as<EXACT, true, true, true> : ppr ? launch_as<EXACT, true, false, true> : launch_as<EXACT, true, false, false>)
+                        : (lab ? launch_as<EXACT, false, true, true> : launch_as<EXACT, false, false, true>);
+    return as(g, reqs, n_req, total, cursor, counters, tu, stream);
 }
 
 template <bool EXACT>
 cudaError_t serve_mode(const GraphDev& g, const ServeDev& sv, Scratch* scratch, const Tuning& tu, cudaStream_t stream) {
-    auto kern = walk_kernel<EXACT, true, true, true>;
+    auto kern = walk_kernel<EXACT, true, true, true, true>;
     // One 768-thread CTA fills an SM (24 warps of 80 registers), so that the
     // eight SMs left out below are wholly free for other streams' kernels.
     // Filling every SM would hold those back for as long as the server runs,
