@@ -39,11 +39,16 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) { retu
 
 // Per-step block: counter (t, q_lo, q_hi, 0), key (seed_lo, seed_hi).
 // Words x|y<<32 give the exact-mode 64-bit draw, word z the PPR stop test.
+template <int UNROLL>
+__host__ __device__ __forceinline__ uint4 step_block_by(uint64_t seed, uint64_t qid, uint32_t t) {
+    return philox4x32_10_by<UNROLL>(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32), 0u),
+                                    make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+}
+
 __host__ __device__ __forceinline__ uint4 step_block(uint64_t seed, uint64_t qid, uint32_t t) {
     // (rolled here and below: the walk engine evaluates one block per step and
     // its loop has to fit the instruction cache)
-    return philox4x32_10_by<1>(make_uint4(t, (uint32_t)qid, (uint32_t)(qid >> 32), 0u),
-                               make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+    return step_block_by<1>(seed, qid, t);
 }
 
 // Fast-mode reservoir draws: counter word 3 = 0x80000000 | lane << 16 | k.
