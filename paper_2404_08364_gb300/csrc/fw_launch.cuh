@@ -75,7 +75,7 @@ cudaError_t launch_as(const GraphDev& g, const ReqTable& reqs, int n_req, int64_
         // per SM would run the rest as a second round (4,800 weighted walks of
         // 80 on R-MAT-22, fast 1,416 us with the large CTAs, 1,152 without).
         // Measured (us): 1,000 exact walks of 80 on a 1,000-vertex graph 617
-        // (four walks per warp) -> 222; 32 node2vec walks of 40 on R-MAT-22,
+        // (four walks per warp) -> 222 (174 with what came later); 32 node2vec walks of 40 on R-MAT-22,
         // fast 868 -> 777, exact 1,095 -> 712 (helpers); 129 PPR walks on
         // R-MAT-22 222 -> 201.
         use = 1;

@@ -474,7 +474,11 @@ __device__ int draw_expj(Group<K>& G, const float* __restrict__ w, int64_t n, ui
 // one chunk or element per thread (SHORT), few (FEW), any number (LONG).  CTAs
 // per SM: the four-chunk race needs 48 registers, a single chunk 40; at CTA
 // width 32 with a few spills are better there, as the barriers want more warps
-// (2^18 draws of 32 weights: 462 us against 533).
+// (2^18 draws of 32 weights: 462 us against 533).  DPRS and ZPRS run on 32
+// throughout; their LONG builds at warp width spill a little for it (52 and 16
+// bytes) and are faster than on 40 without (2^18 draws of 2,000 weights: DPRS
+// 1,051 us against 1,128, ZPRS 727 against 794; only ZPRS at 2^20 weights is
+// slower, 6.98 ms against 6.73 for 4,096 draws).
 enum Form { SHORT, FEW, LONG };
 template <int METHOD, int K, Form FORM>
 __global__ void __launch_bounds__(256, METHOD == SAMP_EXPJ && FORM == LONG   ? 5
